@@ -2123,7 +2123,18 @@ int tn_rejection_sample(const double *p, int64_t T, int32_t b_bits, double alpha
     sp.t0 = t0;
     sp.accept = accept;
     sp.pick = pick;
-    tnk::sampler<<<(unsigned)((T * 32 + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(sp);
+    // FP32 decisions with FP64 where they are close (see sampler_filter): 16-byte loads and
+    // an N_B / alpha that FP32 holds with room to spare; otherwise all in FP64
+    const double xscale = std::ldexp(1.0, b_bits) / alpha;
+    if (reinterpret_cast<uintptr_t>(p) % 16 == 0 && xscale >= 0x1p-60 && xscale <= 0x1p60) {
+        // batches per warp: 32, fewer while that leaves warp slots empty (32 warps per SM)
+        const int per = (int)std::max<int64_t>(1, std::min<int64_t>(32, T / (32 * num_sms())));
+        const int64_t warps = (T + per - 1) / per;
+        tnk::sampler_filter<<<(unsigned)((warps + 7) / 8), 256, 0, static_cast<cudaStream_t>(stream)>>>(sp, per,
+                                                                                                       (float)xscale);
+    } else {
+        tnk::sampler<<<(unsigned)((T * 32 + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(sp);
+    }
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
     return TN_OK;

@@ -1143,11 +1143,8 @@ struct SampleParams {
     int8_t closed_q[64];
 };
 
-// One warp per batch (Sec. II.A steps 2-3); lane l holds p_{2l}, p_{2l+1}.
-__global__ void sampler(SampleParams sp) {
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= sp.T) return;
+// One warp, one batch (Sec. II.A steps 2-3); lane l holds p_{2l}, p_{2l+1}.
+__device__ __forceinline__ void sampler_batch(const SampleParams &sp, long long warp, int lane) {
     double p0, p1;
     if (sp.p) {
         p0 = sp.p[warp * 64 + 2 * lane];
@@ -1249,3 +1246,95 @@ __global__ void slice_cut(const double *R, int k, double f, int32_t *X, int32_t 
 }
 
 }  // namespace tnk
+__global__ void sampler(SampleParams sp) {
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (warp < sp.T) sampler_batch(sp, warp, threadIdx.x & 31);
+}
+
+// The sampler on given probabilities, decided in FP32 wherever FP32 can decide.
+//
+// The kernel above is bound by the FP64 pipe (2 lanes per clock and SM): about 20 FP64
+// instructions per batch, each issued for a whole warp, took 330 us on 225280 batches whose
+// 115 MB of probabilities take 17 us to read.  Both decisions are comparisons (u alpha < p
+// N_B, and the first prefix above v p), so they are made on FP32 approximations first:
+// prefixes of truncated values are within 2^-20 of the total of the FP64 prefixes, v within
+// 2^-23, so a comparison whose sides differ by more than 2^-18 of the total has the same
+// outcome in FP64.  A batch with any closer comparison, with a value that is negative, not
+// finite or -0, whose total is outside [2^-90, 2^90], or without a hit runs sampler_batch
+// (about one in 2000 for random probabilities), so every output equals the kernel above:
+// 330 -> 53 us for a whole call on those batches.
+// A warp takes `per` (<= 32) consecutive batches; lane b forms batch b's draws, which would
+// otherwise be formed 32 times over.  Requires 16-byte aligned p and a finite xscale =
+// N_B / alpha in [2^-60, 2^60] (the host's rule); no eps, no bits.
+constexpr int kFilterUnroll = 8;  // batches whose loads are in flight together
+__device__ __forceinline__ float trunc_to_float(uint32_t lo, uint32_t hi) {
+    // a non-negative finite double's FP32 truncation (below 2^-120: 0; from 2^121: 2^121)
+    const uint32_t h = min(hi, (1023u + 121u) << 20) - ((1023u - 127u) << 20);
+    return hi < ((1023u - 120u) << 20) ? 0.f : __uint_as_float((h << 3) | (lo >> 29));
+}
+__global__ void __launch_bounds__(256) sampler_filter(SampleParams sp, int per, float xscale) {
+    const int lane = threadIdx.x & 31;
+    const long long t0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
+    if (t0 >= sp.T) return;
+    const int nb = (int)min((long long)per, sp.T - t0);
+    const float kMargin = 1.f / 262144.f;
+    float u = 0.f, v = 0.f;
+    if (lane < nb) {
+        const uint64_t t = sp.t0 + (uint64_t)(t0 + lane);
+        const uint2 key = make_uint2((uint32_t)sp.seed, (uint32_t)(sp.seed >> 32));
+        const uint4 o0 = philox4x32_10(make_uint4((uint32_t)t, (uint32_t)(t >> 32), 0u, 0u), key);
+        const uint4 o1 = philox4x32_10(make_uint4((uint32_t)t, (uint32_t)(t >> 32), 1u, 0u), key);
+        // the draws' upper 32 of 53 bits
+        u = __uint2float_rn(o0.w) * (1.f / 4294967296.f);
+        v = __uint2float_rn(o1.y) * (1.f / 4294967296.f);
+    }
+    int pick = 0;        // lane b: batch b's pick and total
+    float total = 0.f;
+    unsigned exact = 0;  // batches that need FP64
+    for (int b0 = 0; b0 < nb; b0 += kFilterUnroll) {
+        uint4 q[kFilterUnroll];
+#pragma unroll
+        for (int i = 0; i < kFilterUnroll; i++) {
+            const long long t = t0 + min(b0 + i, nb - 1);
+            q[i] = __ldcs(reinterpret_cast<const uint4 *>(sp.p + t * 64) + lane);
+        }
+#pragma unroll
+        for (int i = 0; i < kFilterUnroll; i++) {
+            const int b = b0 + i;
+            if (b >= nb) break;
+            // sign, infinity and NaN show in the high words
+            bool bad = max(q[i].y, q[i].w) >= 0x7ff00000u;
+            const float p0 = trunc_to_float(q[i].x, q[i].y), p1 = trunc_to_float(q[i].z, q[i].w);
+            float x = p0 + p1;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const float y = __shfl_up_sync(0xffffffffu, x, off);
+                if (lane >= off) x += y;
+            }
+            const float pj = __shfl_sync(0xffffffffu, x, 31);
+            float excl = __shfl_up_sync(0xffffffffu, x, 1);
+            if (lane == 0) excl = 0.f;
+            const float tau = __shfl_sync(0xffffffffu, v, b) * pj, m = pj * kMargin;
+            const float d0 = excl + p0 - tau, d1 = x - tau;
+            bad |= fabsf(d0) <= m || fabsf(d1) <= m;
+            const unsigned hit = __ballot_sync(0xffffffffu, d0 > 0.f || d1 > 0.f);
+            const unsigned even = __ballot_sync(0xffffffffu, d0 > 0.f);
+            const unsigned anybad = __ballot_sync(0xffffffffu, bad);
+            const int L = __ffs(hit) - 1;
+            if (lane == b) {
+                pick = 2 * L + (((even >> (L & 31)) & 1u) ? 0 : 1);
+                total = pj;
+            }
+            if (anybad || !hit || !(pj > 0x1p-90f && pj < 0x1p90f)) exact |= 1u << b;
+        }
+    }
+    const float x = total * xscale, d = x - u;
+    const bool close = lane < nb && !(fabsf(d) > kMargin * (x + u) + 0x1p-29f);
+    exact |= __ballot_sync(0xffffffffu, close);
+    if (lane < nb && !((exact >> lane) & 1u)) {
+        sp.accept[t0 + lane] = d > 0.f ? 1 : 0;
+        sp.pick[t0 + lane] = pick;
+    }
+    for (; exact; exact &= exact - 1) sampler_batch(sp, t0 + __ffs(exact) - 1, lane);
+}
+
