@@ -2021,32 +2021,34 @@ int tn_slice_cut(const double *R, int32_t k, double f, void *stream, int32_t *X,
     if (!R || !X || !n_x || !F || k < 0 || k > 12) { tn_set_error("tn_slice_cut: bad arguments (k <= 12)"); return TN_EINVAL; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int n = 1 << k;
-    void *buf[4] = {nullptr, nullptr, nullptr, nullptr};
-    const size_t sz[4] = {n * sizeof(double), n * sizeof(int32_t), sizeof(int32_t), sizeof(double)};
-    // every buffer taken is returned to the stream's pool on every exit path
+    // one buffer: the norms, then the results (F, the count, X) as one block to copy back
+    const size_t in_bytes = std::max<size_t>(n * sizeof(double), 16);
+    const size_t out_bytes = 16 + n * sizeof(int32_t);
+    void *buf = nullptr;
+    unsigned char host[16 + 4096 * sizeof(int32_t)];
     auto run = [&]() -> int {
-        for (int i = 0; i < 4; i++) CK(cudaMallocAsync(&buf[i], sz[i], st));
-        double *dR = static_cast<double *>(buf[0]);
-        int32_t *dX = static_cast<int32_t *>(buf[1]), *dn = static_cast<int32_t *>(buf[2]);
-        double *dF = static_cast<double *>(buf[3]);
+        CK(cudaMallocAsync(&buf, in_bytes + out_bytes, st));
+        double *dR = static_cast<double *>(buf);
+        unsigned char *res = static_cast<unsigned char *>(buf) + in_bytes;
         CK(cudaMemcpyAsync(dR, R, n * sizeof(double), cudaMemcpyHostToDevice, st));
         size_t smem = (size_t)n * (sizeof(double) + sizeof(int));
-        tnk::slice_cut<<<1, 256, smem, st>>>(dR, k, f, dX, dn, dF);
+        tnk::slice_cut<<<1, tnk::slice_cut_threads(k), smem, st>>>(dR, k, f, reinterpret_cast<int32_t *>(res + 16),
+                                                                   reinterpret_cast<int32_t *>(res + 8),
+                                                                   reinterpret_cast<double *>(res));
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(n_x, dn, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(F, dF, sizeof(double), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(host, res, out_bytes, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
-        CK(cudaMemcpyAsync(X, dX, (size_t)(*n_x) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        std::memcpy(F, host, sizeof(double));
+        std::memcpy(n_x, host + 8, sizeof(int32_t));
+        std::memcpy(X, host + 16, (size_t)(*n_x) * sizeof(int32_t));
         return TN_OK;
     };
     int rc = run();
-    for (int i = 0; i < 4; i++)
-        if (buf[i] && cudaFreeAsync(buf[i], st) != cudaSuccess && rc == TN_OK) {
-            tn_set_error("tn_slice_cut: cudaFreeAsync failed");
-            rc = TN_EDEVICE;
-        }
-    if (cudaStreamSynchronize(st) != cudaSuccess && rc == TN_OK) {
-        tn_set_error("tn_slice_cut: stream synchronisation failed");
+    // the buffer goes back to the stream's pool on every exit path.  Nothing waits after
+    // that: a wait would hand the pool's memory back to the system, to be mapped again by
+    // the next call
+    if (buf && cudaFreeAsync(buf, st) != cudaSuccess && rc == TN_OK) {
+        tn_set_error("tn_slice_cut: cudaFreeAsync failed");
         rc = TN_EDEVICE;
     }
     return rc;
@@ -2669,7 +2671,7 @@ extern "C" int tn_slice_cut_noalloc(const double *R, int32_t k, double f, void *
     CK(cudaMemsetAsync(b + kCutRBytes + kCutXBytes, 0, 256, st));
     CK(cudaMemcpyAsync(dR, R, n * sizeof(double), cudaMemcpyHostToDevice, st));
     size_t smem = (size_t)n * (sizeof(double) + sizeof(int));
-    tnk::slice_cut<<<1, 256, smem, st>>>(dR, k, f, dX, dn, dF);
+    tnk::slice_cut<<<1, tnk::slice_cut_threads(k), smem, st>>>(dR, k, f, dX, dn, dF);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(n_x, dn, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(F, dF, sizeof(double), cudaMemcpyDeviceToHost, st));

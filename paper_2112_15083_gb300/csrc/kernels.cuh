@@ -1203,49 +1203,6 @@ __device__ __forceinline__ void sampler_batch(const SampleParams &sp, long long 
     }
 }
 
-// ---------------------------------------------------------------- slice cut
-
-// Alg. 1 steps 4-5 for 2^k <= 4096 norms in one block: bitonic sort of (R desc, i asc)
-// in shared memory, then a sequential FP64 prefix in sorted order.
-__global__ void slice_cut(const double *R, int k, double f, int32_t *X, int32_t *n_x, double *F) {
-    extern __shared__ unsigned char smem[];
-    const int n = 1 << k;
-    double *r = reinterpret_cast<double *>(smem);
-    int *idx = reinterpret_cast<int *>(r + n);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) { r[i] = R[i]; idx[i] = i; }
-    __syncthreads();
-    for (int size = 2; size <= n; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    // "before(a, b)": a precedes b in (R descending, index ascending) order
-                    const bool a_first = r[i] > r[j] || (r[i] == r[j] && idx[i] < idx[j]);
-                    const bool up = (i & size) == 0;
-                    if (up != a_first) {
-                        const double tr = r[i]; r[i] = r[j]; r[j] = tr;
-                        const int ti = idx[i]; idx[i] = idx[j]; idx[j] = ti;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    if (threadIdx.x == 0) {
-        double acc = 0.0;
-        int cnt = n;
-        for (int t = 0; t < n; t++) {
-            acc = __dadd_rn(acc, r[t]);
-            if (acc >= f) { cnt = t + 1; break; }
-        }
-        *n_x = cnt;
-        *F = acc;
-    }
-    __syncthreads();
-    const int cnt = *n_x;
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) X[t] = idx[t];
-}
-
-}  // namespace tnk
 __global__ void sampler(SampleParams sp) {
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp < sp.T) sampler_batch(sp, warp, threadIdx.x & 31);
@@ -1338,3 +1295,105 @@ __global__ void __launch_bounds__(256) sampler_filter(SampleParams sp, int per, 
     for (; exact; exact &= exact - 1) sampler_batch(sp, t0 + __ffs(exact) - 1, lane);
 }
 
+// ---------------------------------------------------------------- slice cut
+
+// A double as an unsigned integer in the same order (-0 as +0; NaN as 0, below all others).
+__device__ __forceinline__ unsigned long long order_key(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    if ((b << 1) > 0xffe0000000000000ull) return 0ull;
+    if ((b << 1) == 0ull) return 1ull << 63;
+    return b >> 63 ? ~b : b | (1ull << 63);
+}
+__device__ __forceinline__ double order_value(unsigned long long k) {
+    if (k == 0ull) return __longlong_as_double(0x7ff8000000000000ll);
+    return __longlong_as_double((long long)(k >> 63 ? k & ~(1ull << 63) : ~k));
+}
+
+// Alg. 1 steps 4-5 for 2^k <= 4096 norms in one block: bitonic sort of (R desc, i asc)
+// in shared memory, then a sequential FP64 prefix in sorted order.  Bound by latency.  The
+// sort compares order keys as integers (an FP64 comparison of a whole warp holds the SM's
+// FP64 pipe 16 cycles, and the sort makes up to 2.5 per element and stage); a thread owns
+// pair t of each stage, so the stages with strides up to 32 stay inside a warp's 64
+// elements and need no block barrier (21 barriers instead of 78 at 2^12).  The prefix keeps
+// one FP64 addition per element in its chain: eight values are fetched ahead and the
+// comparisons with f are integer ones.  A whole
+// call at 2^12 norms and f = 0.3: 547 -> 149 us (2^9, f = 1/64: 288 -> 47 us), with one buffer
+// and one copy back instead of four buffers and three copies.
+__global__ void __launch_bounds__(1024) slice_cut(const double *R, int k, double f, int32_t *X, int32_t *n_x, double *F) {
+    extern __shared__ unsigned char smem[];
+    const int n = 1 << k;
+    unsigned long long *r = reinterpret_cast<unsigned long long *>(smem);
+    int *idx = reinterpret_cast<int *>(r + n);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) { r[i] = order_key(R[i]); idx[i] = i; }
+    __syncthreads();
+    for (int size = 2; size <= n; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
+                const int i = ((t & ~(stride - 1)) << 1) | (t & (stride - 1)), j = i | stride;
+                const unsigned long long a = r[i], b = r[j];
+                const int ia = idx[i], ib = idx[j];
+                // i before j in (R descending, index ascending) order; never with a NaN
+                const bool a_first = a != 0 && b != 0 && (a > b || (a == b && ia < ib));
+                if (((i & size) == 0) != a_first) {
+                    r[i] = b;
+                    r[j] = a;
+                    idx[i] = ib;
+                    idx[j] = ia;
+                }
+            }
+            // the next stage's stride (the next size's first one when this is the last)
+            const int next = stride > 1 ? stride >> 1 : size;
+            if (stride > 32 || next > 32) __syncthreads();
+            else __syncwarp();
+        }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned long long fk = f == f ? order_key(f) : ~0ull;  // no sum reaches a NaN f
+        double acc = 0.0;
+        int cnt = n, t = 0;
+        constexpr int U = 8;
+        if (n >= U) {
+            unsigned long long nx[U];
+#pragma unroll
+            for (int i = 0; i < U; i++) nx[i] = r[i];
+            for (; t < n && cnt == n; t += U) {
+                double x[U];
+#pragma unroll
+                for (int i = 0; i < U; i++) x[i] = order_value(nx[i]);
+                if (t + U < n) {
+#pragma unroll
+                    for (int i = 0; i < U; i++) nx[i] = r[t + U + i];
+                }
+                double s[U];
+                s[0] = __dadd_rn(acc, x[0]);
+#pragma unroll
+                for (int i = 1; i < U; i++) s[i] = __dadd_rn(s[i - 1], x[i]);
+                acc = s[U - 1];
+                bool hit = false;
+#pragma unroll
+                for (int i = 0; i < U; i++)
+                    if (!hit && order_key(s[i]) >= fk) {
+                        hit = true;
+                        acc = s[i];
+                        cnt = t + i + 1;
+                    }
+                if (hit) break;
+            }
+        } else {
+            for (; t < n; t++) {
+                acc = __dadd_rn(acc, order_value(r[t]));
+                if (order_key(acc) >= fk) { cnt = t + 1; break; }
+            }
+        }
+        r[0] = (unsigned long long)cnt;  // the sorted keys are no longer needed
+        *n_x = cnt;
+        *F = acc;
+    }
+    __syncthreads();
+    const int cnt = (int)r[0];
+    for (int t = threadIdx.x; t < cnt; t += blockDim.x) X[t] = idx[t];
+}
+// Threads of a slice_cut block: one per pair of a stage, whole warps.
+inline int slice_cut_threads(int k) { return 1 << (k < 6 ? 5 : k > 11 ? 10 : k - 1); }
+
+}  // namespace tnk

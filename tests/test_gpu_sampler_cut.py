@@ -1,5 +1,5 @@
-"""The accept / pick step decided in FP32 against the one decided in FP64.
-"""
+"""The accept / pick step decided in FP32 against the one decided in FP64, and the slice cut
+against a sequential restatement, at the edges of their ranges."""
 import numpy as np
 import pytest
 
@@ -50,3 +50,26 @@ def test_sampler_equals_the_fp64_sampler(T, b_bits, alpha):
     for seed in (1, 2):
         a, b = (P.rejection_sample(x, b_bits, alpha, seed, t0=seed * 1000) for x in (p, q))
         assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("k", [0, 1, 3, 5, 6, 7, 11, 12])
+@pytest.mark.parametrize("f", [1e-9, 0.3, 0.999, 2.0])
+def test_slice_cut_equals_a_sequential_cut(k, f):
+    import paper_2112_15083_gb300 as P
+    rng = np.random.default_rng(100 * k + int(10 * f))
+    R = rng.exponential(size=1 << k)
+    R[rng.random(R.size) < 0.2] = 0.0  # ties, broken by index
+    R /= max(R.sum(), 1e-3)
+    if R.size >= 8:
+        R[3], R[5] = -0.0, -1e-9
+    order = np.lexsort((np.arange(R.size), -R))
+    acc, n = 0.0, R.size
+    for t, i in enumerate(order):
+        acc += R[i]
+        if acc >= f:
+            n = t + 1
+            break
+    X, F = P.slice_cut(R, f)
+    assert np.array_equal(X, order[:n]) and F == acc
+    X, F = P.tn.slice_cut_noalloc(R, f)
+    assert np.array_equal(X, order[:n]) and F == acc
