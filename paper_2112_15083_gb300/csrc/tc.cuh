@@ -302,6 +302,113 @@ struct TcSmem {
 constexpr int kTcEpiWarps = 8;   // two per TMEM lane quarter, each owning half the tile's columns
 constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;  // warp 0: TMA, warp 1: MMA, warps 2-9: epilogue
 
+// 32 bytes (a whole sector) in one store instruction; dst 32-byte aligned.
+__device__ __forceinline__ void st_global_32(void *dst, const uint32_t *w) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                 "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+
+// hi and lo parts of two values as packed 16-bit pairs (the roundings of store_split).
+__device__ __forceinline__ void split_pack2(float a, float b, bool fp16, uint32_t &hi, uint32_t &lo) {
+    if (fp16) {
+        const __half2 h = __floats2half2_rn(a, b);
+        const float2 f = __half22float2(h);
+        const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+        hi = *reinterpret_cast<const uint32_t *>(&h);
+        lo = *reinterpret_cast<const uint32_t *>(&l);
+    } else {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        hi = *reinterpret_cast<const uint32_t *>(&h);
+        const __nv_bfloat162 l =
+            __floats2bfloat162_rn(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+        lo = *reinterpret_cast<const uint32_t *>(&l);
+    }
+}
+
+// How the epilogue's lanes (one tile row each) and their 16 columns lie in C.
+struct TcStorePlan {
+    int nrun;    // 2^nrun columns are adjacent (the columns' lowest bits are C's lowest)
+    bool mpair;  // rows 2 i and 2 i + 1 are adjacent (the rows' lowest bit is C's lowest)
+    bool odd;    // this lane's row is odd
+};
+
+// Store 16 results of one tile row, column j at off0 + lo[j] (elements), if ok; every lane of
+// the warp calls it.  The stores, not the products, set the pace of the tiles with small
+// K: a lane that holds one row of a C with n lowest touches 32 separate sectors per store
+// instruction whatever its width, so its adjacent columns go out together, up to 32 bytes at
+// a time; with m lowest and split planes a 2-byte store per lane fills only 64 bytes per
+// instruction, so neighbouring lanes exchange columns and store two rows of one column as
+// 4 bytes.  (bat, m, n, k bits) = (12, 11, 5, 8), stacked, n lowest, complex64: 2.3 -> 1.95
+// ms; (0, 21, 11, 7), m lowest, split: 15.5 -> 12.1 ms; (0, 23, 7, 5): 3.7 -> 2.75 ms.
+__device__ __forceinline__ void tc_store16(const TcParams &p, void *Cv, long long off0, const long long (&lo)[16],
+                                           const TcStorePlan sp, bool ok, const float (&re)[16], const float (&im)[16]) {
+    const float sc = p.out_scale;
+    if (p.out_fmt == OUT_C64) {
+        if (!ok) return;
+        float2 *c = static_cast<float2 *>(Cv) + off0;
+        if (sp.nrun >= 2) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+                uint32_t w[8];
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    w[2 * i] = __float_as_uint(re[j + i] * sc);
+                    w[2 * i + 1] = __float_as_uint(im[j + i] * sc);
+                }
+                st_global_32(c + lo[j], w);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; j++) c[lo[j]] = make_float2(re[j] * sc, im[j] * sc);
+        }
+        return;
+    }
+    const bool fp16 = p.out_fmt == OUT_SPLIT_FP16;
+    unsigned short *h = static_cast<unsigned short *>(Cv) + off0;
+#pragma unroll
+    for (int ri = 0; ri < 2; ri++) {
+        unsigned short *ph = h + 2 * ri * p.c_plane, *pl = ph + p.c_plane;
+        uint32_t hi[8], lw[8];
+#pragma unroll
+        for (int j = 0; j < 16; j += 2)
+            split_pack2((ri ? im[j] : re[j]) * sc, (ri ? im[j + 1] : re[j + 1]) * sc, fp16, hi[j / 2], lw[j / 2]);
+        if (sp.mpair) {
+            // an even lane keeps column j, its odd neighbour column j + 1
+            const uint32_t sel = sp.odd ? 0x3276u : 0x5410u;
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+                const uint32_t oh = __shfl_xor_sync(0xffffffffu, hi[j / 2], 1);
+                const uint32_t ol = __shfl_xor_sync(0xffffffffu, lw[j / 2], 1);
+                const long long o = sp.odd ? lo[j + 1] - 1 : lo[j];
+                if (ok) {
+                    *reinterpret_cast<uint32_t *>(ph + o) = __byte_perm(hi[j / 2], oh, sel);
+                    *reinterpret_cast<uint32_t *>(pl + o) = __byte_perm(lw[j / 2], ol, sel);
+                }
+            }
+        } else if (!ok) {
+            continue;
+        } else if (sp.nrun >= 4) {
+            st_global_32(ph, hi);
+            st_global_32(pl, lw);
+        } else if (sp.nrun >= 2) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+                *reinterpret_cast<uint2 *>(ph + lo[j]) = make_uint2(hi[j / 2], hi[j / 2 + 1]);
+                *reinterpret_cast<uint2 *>(pl + lo[j]) = make_uint2(lw[j / 2], lw[j / 2 + 1]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+                ph[lo[j]] = (unsigned short)hi[j / 2];
+                ph[lo[j + 1]] = (unsigned short)(hi[j / 2] >> 16);
+                pl[lo[j]] = (unsigned short)lw[j / 2];
+                pl[lo[j + 1]] = (unsigned short)(lw[j / 2] >> 16);
+            }
+        }
+    }
+}
+
 // Persistent kernel: CTA c processes tiles c, c + gridDim.x, ...  Tile order: N tiles
 // fastest, then M tiles, then batch, then explicit version (CTAs running together share
 // the A row panel).  Operand maps are 4-D: [version][4 * BAT planes][rows][K].
@@ -524,6 +631,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (*abort_flag && last_b >= 0) mbar_drain(smem_u32(&acc_full[last_b]), last_par, kLimit);
         }
     } else {
+        TcStorePlan plan = {0, p.lm > 0 && p.pos_m[0] == 0, (row & 1) != 0};
+        while (plan.nrun < lo_bits && p.pos_n[plan.nrun] == plan.nrun) plan.nrun++;
         // epilogue warps 2..9: TMEM lane quarter = warp % 4 = tile rows 32*(warp%4)..; warps
         // 2-5 store columns [0, BN/2) of the tile, warps 6-9 columns [BN/2, BN)
         const int quarter = warp & 3;
@@ -536,7 +645,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int j = 0; j < 16; j++) lo[j] = scatter_bits(j, p.pos_n, lo_bits);
         int it = 0;
-        for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
+        for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
             const int b = it & 1;
             // the tile's coordinates and output bases first: their loads and bit scatters
             // overlap the wait for the accumulator
@@ -589,28 +698,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (be < 0) continue;
                 __syncwarp();
                 tmem_ld16x2(lane_addr + c0, lane_addr + BN + c0, re, im);
-                if (!row_ok) continue;
-                if (stk) {
-                    const long long cb = first ? cb0 : cb1;
-                    const long long nb = c0 & (N - 1);
-                    void *Cv = static_cast<char *>(p.C) + 8 * vrow * p.c_plane;
-                    const long long hi = cb + scatter_bits(nb >> 4, p.pos_n + 4, p.ln - 4);
+                if (p.ln < 4) {
+                    if (!row_ok) continue;
+                    // fewer than 16 columns per version: versions folded into N, column by
+                    // column (c0 + j is column n of version v)
 #pragma unroll
                     for (int j = 0; j < 16; j++) {
-                        const long long off = hi + lo[j];
-                        const float2 x = make_float2(re[j] * p.out_scale, im[j] * p.out_scale);
-                        if (p.out_fmt == OUT_C64) static_cast<float2 *>(Cv)[off] = x;
-                        else store_split(Cv, p.c_plane, off, x, p.out_fmt == OUT_SPLIT_FP16);
-                    }
-                    continue;
-                }
-                if (p.fold == 2) {
-                    // columns: version (c0 + j) / N of this tile, n = (c0 + j) % N
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const long long col = c0 + j;
-                        const long long v = (long long)tn_i * vn + (col >> p.ln), n = col & (N - 1);
-                        if (v < p.nver) {
+                        const long long col = (long long)tn_i * BN + c0 + j;
+                        const long long v = vrow + (col >> p.ln), n = col & (N - 1);
+                        if (v < p.nver && (p.fold == 2 || col < N)) {
                             void *Cv = static_cast<char *>(p.C) + 8 * v * p.c_plane;
                             const long long off = cbase + scatter_bits(n, p.pos_n, p.ln);
                             const float2 x = make_float2(re[j] * p.out_scale, im[j] * p.out_scale);
@@ -619,20 +715,19 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         }
                     }
                     continue;
+                tc_store16(p, static_cast<char *>(p.C) + 8 * v * p.c_plane,
+                           hi + scatter_bits(nb >> 4, p.pos_n + 4, p.ln - 4), lo, plan, row_ok && nb < N && v < p.nver,
+                           re, im);
                 }
-                void *Cv = static_cast<char *>(p.C) + 8 * vrow * p.c_plane;
-                const long long nb = (long long)tn_i * BN + c0;
-                if (nb < N) {
-                    const long long hi = cbase + (p.ln > 4 ? scatter_bits(nb >> 4, p.pos_n + 4, p.ln - 4) : 0);
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        if (nb + j < N) {
-                            const long long off = hi + lo[j];
-                            const float2 x = make_float2(re[j] * p.out_scale, im[j] * p.out_scale);
-                            if (p.out_fmt == OUT_C64) static_cast<float2 *>(Cv)[off] = x;
-                            else store_split(Cv, p.c_plane, off, x, p.out_fmt == OUT_SPLIT_FP16);
-                        }
-                    }
+                // 16 columns of one batch and version: column nb + j at hi + lo[j]
+                const long long col = (long long)tn_i * BN + c0;
+                long long v = vrow, nb = col, hi = cbase;
+                if (stk) {
+                    hi = first ? cb0 : cb1;
+                    nb = c0 & (N - 1);
+                } else if (p.fold == 2) {
+                    v = col >> p.ln;
+                    nb = col & (N - 1);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
