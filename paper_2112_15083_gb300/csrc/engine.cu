@@ -996,10 +996,7 @@ int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
             };
             auto by_n = [&](auto m_tag) {
                 constexpr int M = decltype(m_tag)::value;
-                // two rows per warp: 32-row blocks get 16 warps, enough to keep the FMA pipe
-                // fed (4096 batches of 64 x 8 outputs over K = 2048: 1.58 ms, against 2.0 ms
-                // with 8 warps of four rows and 1.95 ms with 32 warps of one row)
-                constexpr int W = M >= 2 ? M / 2 : 1, MW = M / W;
+                constexpr int MW = M >= 4 ? 4 : M, W = M / MW;
                 switch (p.ln) {
                     case 0: go(tnk::cgemm_skinny<W, MW, 1>, W, tnk::skinny_stage_bytes<W, MW, 1>()); break;
                     case 1: go(tnk::cgemm_skinny<W, MW, 2>, W, tnk::skinny_stage_bytes<W, MW, 2>()); break;

@@ -382,20 +382,26 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
 }
 
 // Batched products with at most 64 rows and 8 columns and a long K (K >= 1024, complex64
-// operands).  A block of W warps takes R = W MW rows of one (version, batch) at a time (a
-// batch with more rows is split into row blocks); each warp owns MW rows of A and every
-// column.  The block's work is one sequence of stages, each a (unit, K block of 64 U
-// elements) pair, streamed through a ring of ST shared-memory stages by the bulk-copy
-// engine (one contiguous copy per row and stage, issued ST - 1 stages ahead across unit
-// boundaries and completing on the stage's mbarrier), so loads stay in flight while the
-// FMAs run.  In a stage lane l reads elements 2 l and 2 l + 1 of each 64-element block of
-// its warp's A rows; the stage's B rows are shared by the block.  Every wait is bounded:
-// on timeout the block sets *err, lets its copies in flight land (bounded) and returns.
-// Each lane accumulates in ascending k and the warp adds its 32 lane sums by a fixed xor
-// butterfly.  Gathered operands are read in place, one decode per row and warp.  The lane
-// split of K rounds differently from the kernels that accumulate each output over k in
-// one thread, so it is the only kernel the engine runs for these shapes.
-constexpr int kSkinnyU = 2;   // 64-element K blocks per stage
+// operands).  A block takes R = W MW rows of one (version, batch) at a time (a batch with
+// more rows is split into row blocks); each of W warps owns MW rows of A and every column.
+// The block's work is one sequence of stages, each a (unit, K block of 64 U elements) pair.
+// Warp 0 streams them through a ring of ST shared-memory stages with the bulk-copy engine
+// (one contiguous copy per row and stage, ST - 1 stages ahead across unit boundaries,
+// completing on the stage's `full` barrier); every warp waits for a stage and releases it
+// on its `empty` barrier by itself, so no block barrier ties the warps together.  In a stage
+// lane l reads elements 2 l and 2 l + 1 of each
+// 64-element block of its warp's A rows; the stage's B rows are shared by the block.  Each
+// lane accumulates in ascending k and the warp adds its 32 lane sums in the tree of a xor
+// butterfly (halving the values a lane still holds at each level: 62 shuffles for 32 outputs
+// instead of 320).  Gathered operands are read in place, one decode per row and unit.  Every
+// wait is bounded: on timeout the block sets *err, lets its copies in flight land (bounded)
+// and returns.  The lane split of K rounds differently from the kernels that accumulate
+// each output over k in one thread, so it is the only kernel the engine runs for these
+// shapes.  Bound by shared-memory reads next to FP32 issue: with MW rows a warp reads MW + N
+// 16-byte rows per 8 MW N multiply-adds, so MW is four: (bat, m, n, k bits) =
+// (14, 4, 3, 10) took 1.04 ms with two rows per warp and two block barriers per stage, 0.79 ms
+// so (2.7 TB/s; its 2.2 GB take 0.32 ms at the copy rate).
+constexpr int kSkinnyU = 1;   // 64-element K blocks per stage
 constexpr int kSkinnyST = 4;  // ring stages
 template <int W, int MW, int N>
 constexpr int skinny_stage_bytes() {
@@ -404,9 +410,10 @@ constexpr int skinny_stage_bytes() {
 template <int W, int MW, int N>
 __global__ void __launch_bounds__(32 * W) cgemm_skinny(GemmParams p) {
     extern __shared__ float4 skinny_ring[];
-    __shared__ __align__(8) uint64_t full[kSkinnyST];  // per stage: W arrivals + the bytes
+    constexpr int R = W * MW, U = kSkinnyU, ST = kSkinnyST;
+    constexpr int RPL = (R + N + 31) / 32;  // rows copied per lane of warp 0
+    __shared__ __align__(8) uint64_t full[ST], empty[ST];
     __shared__ int abort_flag;
-    constexpr int R = W * MW, U = kSkinnyU, ST = kSkinnyST, NB = (N + W - 1) / W;
     const long long kLimit = 4000000000LL;
     constexpr int kStage = (R + N) * U * 32;  // float4 per stage
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -414,139 +421,128 @@ __global__ void __launch_bounds__(32 * W) cgemm_skinny(GemmParams p) {
     const long long units = (p.nver << p.lbat) * row_blocks;
     const int nk = (1 << p.lk) / (64 * U);  // stages per unit
     const long long mine = units > blockIdx.x ? (units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const long long total = mine * nk;
-    // copy side: the row pointers of the unit being issued
-    const float2 *a[MW], *b[NB];
-    long long a_unit = -1;
     auto unit_of = [&](long long ul, long long &bat, long long &v, int &row0) {
         const long long u = blockIdx.x + ul * gridDim.x;
-        const int rb = (int)(u % row_blocks);
         const long long bv = u / row_blocks;
         bat = bv & ((1LL << p.lbat) - 1);
         v = bv >> p.lbat;
-        row0 = rb * R + warp * MW;  // this warp's first row of A
+        row0 = (int)(u % row_blocks) * R;  // the unit's first row of A
     };
-    // copies of stage (unit ul, K block kb) into ring slot `slot`
-    auto issue = [&](long long ul, int kb, int slot) {
-        if (ul != a_unit) {
-            long long bat, v;
-            int row0;
-            unit_of(ul, bat, v, row0);
-#pragma unroll
-            for (int i = 0; i < MW; i++) {
-                const long long e = ((bat << p.lm) | (long long)(row0 + i)) << p.lk;
-                a[i] = p.gA ? reinterpret_cast<const float2 *>(p.gA->src) +
-                                  gather_src_warp(*p.gA, e, p.gA->pos_beta[p.gA->lb - 1], p.closed_bits)
-                            : static_cast<const float2 *>(p.ptrA[v]) + e;
-            }
-#pragma unroll
-            for (int r = 0; r < NB; r++) {
-                const int n = warp + r * W;
-                const long long e = (bat << (p.ln + p.lk)) | ((long long)(n < N ? n : 0) << p.lk);
-                b[r] = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) +
-                                  gather_src_warp(*p.gB, e, p.gB->pos_beta[p.gB->lb - 1], p.closed_bits)
-                            : static_cast<const float2 *>(p.ptrB[v]) + e;
-            }
-            a_unit = ul;
-        }
-        // lane 0 of each warp: one arrival with the warp's bytes, then its rows' copies
-        if (lane == 0) {
-            float4 *st = skinny_ring + slot * kStage;
-            const uint32_t bar = smem_u32(&full[slot]);
-            int rows = MW;
-#pragma unroll
-            for (int r = 0; r < NB; r++) rows += warp + r * W < N;
-            mbar_expect_tx(bar, (uint32_t)(rows * U * 512));
-            const int k0 = kb * 64 * U;
-#pragma unroll
-            for (int i = 0; i < MW; i++) bulk_load(&st[(warp * MW + i) * U * 32], a[i] + k0, U * 512, bar);
-#pragma unroll
-            for (int r = 0; r < NB; r++)
-                if (warp + r * W < N) bulk_load(&st[(R + warp + r * W) * U * 32], b[r] + k0, U * 512, bar);
-        }
-    };
-    float2 acc[MW][N];
-#pragma unroll
-    for (int i = 0; i < MW; i++)
-#pragma unroll
-        for (int n = 0; n < N; n++) acc[i][n] = make_float2(0.f, 0.f);
     if (threadIdx.x == 0) {
-        for (int i = 0; i < ST; i++) mbar_init(smem_u32(&full[i]), W);
+        for (int i = 0; i < ST; i++) {
+            mbar_init(smem_u32(&full[i]), 1);
+            mbar_init(smem_u32(&empty[i]), W);
+        }
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    // stage counters advance by one (no divisions in the loop): issue side (iul, ikb, islot)
-    // runs ST - 1 stages ahead of the compute side (ul, kb, slot, parity)
-    long long issued = 0, iul = 0;
+    // warp 0's copy side: stage (iul, ikb) goes to slot islot; lane r copies row r of a stage (A
+    // rows, then B rows), and row r + 32 if there is one
+    const float2 *src[RPL];
+    long long iul = 0, issued = 0;
     int ikb = 0, islot = 0;
-    auto advance_issue = [&]() {
+    uint32_t iparity = 0;
+    auto issue = [&]() {
+        if (iul >= mine) return true;
+        if (ikb == 0) {
+            long long bat, v;
+            int row0;
+            unit_of(iul, bat, v, row0);
+#pragma unroll
+            for (int i = 0; i < RPL; i++) {
+                const int r = lane + 32 * i;
+                if (r < R) {
+                    const long long e = ((bat << p.lm) | (long long)(row0 + r)) << p.lk;
+                    src[i] = p.gA ? reinterpret_cast<const float2 *>(p.gA->src) + gather_src(*p.gA, e, p.closed_bits)
+                                  : static_cast<const float2 *>(p.ptrA[v]) + e;
+                } else if (r < R + N) {
+                    const long long e = ((bat << p.ln) | (long long)(r - R)) << p.lk;
+                    src[i] = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, e, p.closed_bits)
+                                  : static_cast<const float2 *>(p.ptrB[v]) + e;
+                }
+            }
+        }
+        int go = 1;
+        if (lane == 0) {
+            if (issued >= ST) go = mbar_wait(smem_u32(&empty[islot]), iparity ^ 1u, &abort_flag, kLimit);
+            if (go) mbar_expect_tx(smem_u32(&full[islot]), (uint32_t)((R + N) * U * 512));
+        }
+        if (!__shfl_sync(0xffffffffu, go, 0)) return false;
+#pragma unroll
+        for (int i = 0; i < RPL; i++) {
+            const int r = lane + 32 * i;
+            if (r < R + N)
+                bulk_load(&skinny_ring[islot * kStage + r * U * 32], src[i] + ikb * 64 * U, U * 512,
+                          smem_u32(&full[islot]));
+        }
         issued++;
         if (++ikb == nk) { ikb = 0; iul++; }
-        if (++islot == ST) islot = 0;
+        if (++islot == ST) { islot = 0; iparity ^= 1u; }
+        return true;
     };
-    for (; issued < ST - 1 && issued < total;) {
-        issue(iul, ikb, islot);
-        advance_issue();
-    }
-    long long g = 0, ul = 0;
-    int kb = 0, slot = 0;
-    uint32_t parity = 0;
-    for (; g < total; g++) {
-        __syncthreads();  // every warp is done with the slot the next issue overwrites
-        if (issued < total) {
-            issue(iul, ikb, islot);
-            advance_issue();
-        }
-        mbar_wait(smem_u32(&full[slot]), parity, &abort_flag, kLimit);
-        __syncthreads();  // a timeout anywhere ends the block's loop in every thread
-        if (abort_flag) break;
-        const float4 *st = skinny_ring + slot * kStage;
-        if (++slot == ST) { slot = 0; parity ^= 1u; }
+    if (warp == 0)
+        for (int i = 0; i < ST - 1; i++) issue();
+    {
+        int slot = 0;
+        uint32_t parity = 0;
+        bool ok = true;
+        for (long long ul = 0; ul < mine && ok; ul++) {
+            float2 acc[MW * N];
 #pragma unroll
-        for (int u = 0; u < U; u++)
+            for (int o = 0; o < MW * N; o++) acc[o] = make_float2(0.f, 0.f);
+            for (int kb = 0; kb < nk; kb++) {
+                // the slot that warp 0 refills here was read one stage ago
+                if (warp == 0 && !issue()) { ok = false; break; }
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[slot]), parity, &abort_flag, kLimit));
+                if (!ok) break;
+                const float4 *st = skinny_ring + slot * kStage;
 #pragma unroll
-            for (int n = 0; n < N; n++) {
-                const float4 yb = st[((R + n) * U + u) * 32 + lane];
+                for (int u = 0; u < U; u++) {
+                    float4 x[MW];
 #pragma unroll
-                for (int i = 0; i < MW; i++) {
-                    const float4 x = st[((warp * MW + i) * U + u) * 32 + lane];
-                    acc[i][n] = cfma(make_float2(x.x, x.y), make_float2(yb.x, yb.y), acc[i][n]);
-                    acc[i][n] = cfma(make_float2(x.z, x.w), make_float2(yb.z, yb.w), acc[i][n]);
+                    for (int i = 0; i < MW; i++) x[i] = st[((warp * MW + i) * U + u) * 32 + lane];
+#pragma unroll
+                    for (int n = 0; n < N; n++) {
+                        const float4 y = st[((R + n) * U + u) * 32 + lane];
+#pragma unroll
+                        for (int i = 0; i < MW; i++) {
+                            acc[i * N + n] = cfma(make_float2(x[i].x, x[i].y), make_float2(y.x, y.y), acc[i * N + n]);
+                            acc[i * N + n] = cfma(make_float2(x[i].z, x[i].w), make_float2(y.z, y.w), acc[i * N + n]);
+                        }
+                    }
                 }
             }
-        if (++kb < nk) continue;
-        kb = 0;
-        // the unit's last stage: reduce, store, start the next unit from zero
+            if (!ok) break;
+            // add the lanes' sums: at each level a lane keeps the half of the outputs that its
+            // lane bit selects, until it holds one (then both lanes of a pair add the same)
+            int left = MW * N, out = 0;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1)
+            for (int off = 16; off > 0; off >>= 1) {
+                const bool up = (lane & off) != 0;
+                if (left > 1) {
+                    left >>= 1;
+                    out = 2 * out + (up ? 1 : 0);
 #pragma unroll
-            for (int i = 0; i < MW; i++)
-#pragma unroll
-                for (int n = 0; n < N; n++) {
-                    acc[i][n].x += __shfl_xor_sync(0xffffffffu, acc[i][n].x, off);
-                    acc[i][n].y += __shfl_xor_sync(0xffffffffu, acc[i][n].y, off);
+                    for (int o = 0; o < MW * N / 2; o++) {
+                        if (o >= left) break;
+                        const float2 keep = up ? acc[o + left] : acc[o], send = up ? acc[o] : acc[o + left];
+                        acc[o].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, off);
+                        acc[o].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, off);
+                    }
+                } else {
+                    acc[0].x += __shfl_xor_sync(0xffffffffu, acc[0].x, off);
+                    acc[0].y += __shfl_xor_sync(0xffffffffu, acc[0].y, off);
                 }
-        long long bat, v;
-        int row0;
-        unit_of(ul++, bat, v, row0);
-        // every lane holds the totals: lane i N + n stores output (row MW warp + i, column n)
-        const long long cb = scatter_bits(bat, p.pos_bat, p.lbat);
-#pragma unroll
-        for (int i = 0; i < MW; i++)
-#pragma unroll
-            for (int n = 0; n < N; n++) {
-                if (lane == i * N + n)
-                    store_c(p, v, cb + scatter_bits(row0 + i, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln),
-                            acc[i][n]);
-                acc[i][n] = make_float2(0.f, 0.f);
             }
     }
-    if (abort_flag && threadIdx.x == 0) {
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_flag) {
+        // after a timeout, let the copies already issued land before the shared memory is released
         atomicExch(p.err, 1);
-        // let the copies already issued land before the shared memory is released
-        for (long long q = g; q < issued; q++) mbar_drain(smem_u32(&full[q % ST]), (uint32_t)((q / ST) & 1), kLimit);
+        for (long long q = issued > ST ? issued - ST : 0; q < issued; q++)
+            mbar_drain(smem_u32(&full[q % ST]), (uint32_t)((q / ST) & 1), kLimit);
     }
     __syncthreads();
 }
@@ -568,6 +564,10 @@ __global__ void __launch_bounds__(256) cgemm_small(GemmParams p, SmallMap smp) {
     __shared__ SmallMap sm;  // its tables are read per output
     if (threadIdx.x == 0) sm = smp;
     T *As = reinterpret_cast<T *>(small_smem);
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[slot])) : "memory");
+                if (++slot == ST) { slot = 0; parity ^= 1u; }
     const int M = 1 << p.lm, N = 1 << p.ln, K = 1 << p.lk, G = 1 << smp.lg;
     const int KP = K + 1;  // padded row: rows of consecutive outputs fall in different banks
     T *Bs = As + (size_t)G * M * KP;
@@ -595,6 +595,16 @@ __global__ void __launch_bounds__(256) cgemm_small(GemmParams p, SmallMap smp) {
         T acc = czero<T>();
         for (int k = 0; k < K; k++) acc = cfma(a[k], bb[k], acc);
         const long long off = cbase + scatter_bits(b, p.pos_bat, smp.lg) + scatter_bits(m, p.pos_m, p.lm) +
+            if ((lane & (32 / (MW * N) - 1)) == 0) {
+                long long bat, v;
+                int row0;
+                unit_of(ul, bat, v, row0);
+                const int m = row0 + warp * MW + out / N, n = out % N;
+                store_c(p, v,
+                        scatter_bits(bat, p.pos_bat, p.lbat) + scatter_bits(m, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln),
+                        acc[0]);
+            }
+        }
                               scatter_bits(n, p.pos_n, p.ln);
         store_c_t<T>(p, v, off, acc);
     }
