@@ -513,6 +513,10 @@ __global__ void __launch_bounds__(32 * W) cgemm_skinny(GemmParams p) {
                         }
                     }
                 }
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[slot])) : "memory");
+                if (++slot == ST) { slot = 0; parity ^= 1u; }
             }
             if (!ok) break;
             // add the lanes' sums: at each level a lane keeps the half of the outputs that its
@@ -536,6 +540,16 @@ __global__ void __launch_bounds__(32 * W) cgemm_skinny(GemmParams p) {
                     acc[0].y += __shfl_xor_sync(0xffffffffu, acc[0].y, off);
                 }
             }
+            if ((lane & (32 / (MW * N) - 1)) == 0) {
+                long long bat, v;
+                int row0;
+                unit_of(ul, bat, v, row0);
+                const int m = row0 + warp * MW + out / N, n = out % N;
+                store_c(p, v,
+                        scatter_bits(bat, p.pos_bat, p.lbat) + scatter_bits(m, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln),
+                        acc[0]);
+            }
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) {
@@ -564,10 +578,6 @@ __global__ void __launch_bounds__(256) cgemm_small(GemmParams p, SmallMap smp) {
     __shared__ SmallMap sm;  // its tables are read per output
     if (threadIdx.x == 0) sm = smp;
     T *As = reinterpret_cast<T *>(small_smem);
-                __syncwarp();
-                if (lane == 0)
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[slot])) : "memory");
-                if (++slot == ST) { slot = 0; parity ^= 1u; }
     const int M = 1 << p.lm, N = 1 << p.ln, K = 1 << p.lk, G = 1 << smp.lg;
     const int KP = K + 1;  // padded row: rows of consecutive outputs fall in different banks
     T *Bs = As + (size_t)G * M * KP;
@@ -595,16 +605,6 @@ __global__ void __launch_bounds__(256) cgemm_small(GemmParams p, SmallMap smp) {
         T acc = czero<T>();
         for (int k = 0; k < K; k++) acc = cfma(a[k], bb[k], acc);
         const long long off = cbase + scatter_bits(b, p.pos_bat, smp.lg) + scatter_bits(m, p.pos_m, p.lm) +
-            if ((lane & (32 / (MW * N) - 1)) == 0) {
-                long long bat, v;
-                int row0;
-                unit_of(ul, bat, v, row0);
-                const int m = row0 + warp * MW + out / N, n = out % N;
-                store_c(p, v,
-                        scatter_bits(bat, p.pos_bat, p.lbat) + scatter_bits(m, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln),
-                        acc[0]);
-            }
-        }
                               scatter_bits(n, p.pos_n, p.ln);
         store_c_t<T>(p, v, off, acc);
     }

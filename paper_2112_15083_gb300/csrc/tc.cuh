@@ -299,9 +299,6 @@ struct TcSmem {
     static constexpr int kBytes = STAGES * kStage + 1024 /*barriers*/ + 1024 /*alignment*/;
 };
 
-constexpr int kTcEpiWarps = 8;   // two per TMEM lane quarter, each owning half the tile's columns
-constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;  // warp 0: TMA, warp 1: MMA, warps 2-9: epilogue
-
 // 32 bytes (a whole sector) in one store instruction; dst 32-byte aligned.
 __device__ __forceinline__ void st_global_32(void *dst, const uint32_t *w) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
@@ -408,6 +405,9 @@ __device__ __forceinline__ void tc_store16(const TcParams &p, void *Cv, long lon
         }
     }
 }
+
+constexpr int kTcEpiWarps = 8;   // two per TMEM lane quarter, each owning half the tile's columns
+constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;  // warp 0: TMA, warp 1: MMA, warps 2-9: epilogue
 
 // Persistent kernel: CTA c processes tiles c, c + gridDim.x, ...  Tile order: N tiles
 // fastest, then M tiles, then batch, then explicit version (CTAs running together share
@@ -631,8 +631,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (*abort_flag && last_b >= 0) mbar_drain(smem_u32(&acc_full[last_b]), last_par, kLimit);
         }
     } else {
-        TcStorePlan plan = {0, p.lm > 0 && p.pos_m[0] == 0, (row & 1) != 0};
-        while (plan.nrun < lo_bits && p.pos_n[plan.nrun] == plan.nrun) plan.nrun++;
         // epilogue warps 2..9: TMEM lane quarter = warp % 4 = tile rows 32*(warp%4)..; warps
         // 2-5 store columns [0, BN/2) of the tile, warps 6-9 columns [BN/2, BN)
         const int quarter = warp & 3;
@@ -644,6 +642,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         long long lo[16];
 #pragma unroll
         for (int j = 0; j < 16; j++) lo[j] = scatter_bits(j, p.pos_n, lo_bits);
+        TcStorePlan plan = {0, p.lm > 0 && p.pos_m[0] == 0, (row & 1) != 0};
+        while (plan.nrun < lo_bits && p.pos_n[plan.nrun] == plan.nrun) plan.nrun++;
         int it = 0;
         for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
             const int b = it & 1;
@@ -715,9 +715,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         }
                     }
                     continue;
-                tc_store16(p, static_cast<char *>(p.C) + 8 * v * p.c_plane,
-                           hi + scatter_bits(nb >> 4, p.pos_n + 4, p.ln - 4), lo, plan, row_ok && nb < N && v < p.nver,
-                           re, im);
                 }
                 // 16 columns of one batch and version: column nb + j at hi + lo[j]
                 const long long col = (long long)tn_i * BN + c0;
@@ -729,6 +726,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     v = col >> p.ln;
                     nb = col & (N - 1);
                 }
+                tc_store16(p, static_cast<char *>(p.C) + 8 * v * p.c_plane,
+                           hi + scatter_bits(nb >> 4, p.pos_n + 4, p.ln - 4), lo, plan, row_ok && nb < N && v < p.nver,
+                           re, im);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
