@@ -670,7 +670,9 @@ bool stack_fits(const CNet &cn, size_t si, int BN) {
 bool rowstage_fits(const CNet &cn, const Step &s) {
     return cn.elem == 8 && std::min(s.nm, s.nn) <= 5 && s.nk >= 4 && s.nk <= 6;
 }
-constexpr int kTiles[7][2] = {{128, 64}, {64, 64}, {128, 32}, {64, 32}, {32, 32}, {128, 16}, {16, 16}};
+// FFMA tiles (rows x columns); the longer side of a step are the rows.
+constexpr int kTiles[10][2] = {{128, 64}, {64, 64}, {128, 32}, {64, 32}, {32, 32},
+                               {256, 16}, {128, 16}, {256, 8}, {256, 4}, {16, 16}};
 
 // Whether the long-K kernel runs step si: at most 8 outputs on the short side and 64 on
 // the long side, K >= 1024, complex64 operands.  It is then the step's only kernel (its
@@ -703,7 +705,8 @@ std::vector<int> step_variants(const CNet &cn, size_t si) {
     if (rowstage_fits(cn, s)) v.push_back(kVarRowStage);
     if (small_fits(s, (size_t)cn.elem)) v.push_back(kVarSmall);
     for (auto &t : kTiles)
-        if (t[0] == 16 || ((2LL << s.nm) >= t[0] && (2LL << s.nn) >= t[1])) v.push_back(t[0] * 1000 + t[1]);
+        if (t[0] == 16 || ((2LL << std::max(s.nm, s.nn)) >= t[0] && (2LL << std::min(s.nm, s.nn)) >= t[1]))
+            v.push_back(t[0] * 1000 + t[1]);
     return v;
 }
 
@@ -719,12 +722,15 @@ int default_variant(const CNet &cn, size_t si) {
     }
     if (std::min(s.nm, s.nn) == 6 && std::max(s.nm, s.nn) == 6 && small_fits(s, (size_t)cn.elem)) return kVarSmall;
     if (std::min(s.nm, s.nn) <= 5 && s.nk <= 6) return kVarRow;
-    // large products: 128 x 32 tiles (the autotuner's choice on GB300 for complex64)
-    if (s.nm >= 7 && s.nn >= 5) return 128032;
-    if (s.nm >= 6 && s.nn >= 6) return 64064;
-    if (s.nm >= 6 && s.nn >= 5) return 64032;
-    if (s.nm >= 5 && s.nn >= 5) return 32032;
-    if (s.nm >= 7) return 128016;
+    // the largest tile that both sides fill
+    const int lo = std::min(s.nm, s.nn), hi = std::max(s.nm, s.nn);
+    if (lo >= 6 && hi >= 7) return 128064;
+    if (lo >= 5 && hi >= 7) return 128032;
+    if (lo >= 6) return 64064;
+    if (lo >= 5 && hi >= 6) return 64032;
+    if (lo >= 5) return 32032;
+    if (lo == 4 && hi >= 7) return hi >= 8 ? 256016 : 128016;
+    if (hi >= 8) return lo == 3 ? 256008 : 256004;
     return 16016;
 }
 
@@ -748,6 +754,20 @@ bool row_fuses(const CNet &cn, size_t si) {
     return true;
 }
 
+// The complex64 tile kernel reads the gathered operands of step si in place when each one is
+// a single complex version whose batch blocks are contiguous in its source.
+bool tile_fuses(const CNet &cn, size_t si) {
+    const Step &s = cn.steps[si];
+    if (cn.elem != 8 || !(s.gat[0] || s.gat[1]) || cn.cp.gd_off.size() <= si + 1) return false;
+    for (int o = 0; o < 2; o++) {
+        if (!s.gat[o]) continue;
+        const tnk::GatherDesc &g = cn.cp.gd[cn.cp.gd_off[si] + (o == 1 && s.gat[0] ? 1 : 0)];
+        if (g.nver != 1 || g.nplanes != 1 || g.esize != cn.elem || g.lb < 1) return false;
+        if (g.pos_beta[g.lb - 1] < s.nk + (o ? s.nn : s.nm)) return false;
+    }
+    return true;
+}
+
 // The long-K kernel reads a gathered operand in place when it is a single complex version
 // whose every row (K elements) is contiguous in its source.
 bool skinny_fuses(const CNet &cn, size_t si) {
@@ -766,6 +786,7 @@ bool skinny_fuses(const CNet &cn, size_t si) {
 bool reads_in_place(const CNet &cn, size_t si, int var) {
     if (var == kVarRow || var == kVarRowStage) return row_fuses(cn, si);
     if (var == kVarSkinny) return skinny_fuses(cn, si);
+    if (var >= 16000 && !is_tc_variant(var)) return tile_fuses(cn, si);
     if (is_tc_variant(var)) {
         const Step &s = cn.steps[si];
         if (!(s.gat[0] || s.gat[1]) || cn.cp.tc_inplace.size() <= si) return false;
@@ -880,12 +901,11 @@ int step_params(const CNet &cn, const Step &s, tnk::GemmParams &p) {
     return TN_OK;
 }
 
-// The row kernel's roles: one thread per row of the larger side, the small side in
-// registers (C = A B^T is symmetric in the operand roles); gathered operands read in
-// place when possible.
-void row_roles(const CNet &cn, const Step &s, tnk::GemmParams &p) {
+// The roles of the row and tile kernels: the larger side are the rows (C = A B^T is
+// symmetric in the operand roles); gathered operands read in place if `in_place`.
+void row_roles(const CNet &cn, const Step &s, tnk::GemmParams &p, bool in_place) {
     const size_t si = &s - cn.steps.data();
-    if (row_fuses(cn, si) && cn.cur_closed) {
+    if (in_place && cn.cur_closed) {
         const auto *gd = static_cast<const tnk::GatherDesc *>(cn.gdescs.p) + cn.cp.gd_off[si];
         p.gA = s.gat[0] ? gd : nullptr;
         p.gB = s.gat[1] ? gd + (s.gat[0] ? 1 : 0) : nullptr;
@@ -941,7 +961,7 @@ int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
     } else if (var == kVarRowStage) {
         if (!rowstage_fits(cn, s)) { tn_set_error("staged row kernel: unsupported step shape"); return TN_EINVAL; }
         if constexpr (sizeof(T) == sizeof(float2)) {
-            row_roles(cn, s, p);
+            row_roles(cn, s, p, row_fuses(cn, si));
             const long long rows = p.nver << (p.lbat + p.lm);
             const int per_block = 32 * tnk::kRowWarps;
             const size_t smem = (size_t)per_block * (8 * (1 << p.lk) + tnk::kRowPad);
@@ -1018,7 +1038,7 @@ int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
             return TN_EINVAL;
         }
     } else if (var == kVarRow) {
-        row_roles(cn, s, p);
+        row_roles(cn, s, p, row_fuses(cn, si));
         long long rows = p.nver << (p.lbat + p.lm);
         // grid-stride: at most 16 resident blocks' worth per SM, each thread several rows
         unsigned blocks = (unsigned)std::min<long long>((rows + 255) / 256, 16LL * num_sms());
@@ -1031,22 +1051,44 @@ int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
             default: tnk::cgemm_row<T, 32><<<blocks, 256, 0, st>>>(p); break;
         }
     } else {
-        auto launch = [&](auto kern, int TM, int TN) {
-            int ltm = std::min(s.nm, __builtin_ctz(TM)), ltn = std::min(s.nn, __builtin_ctz(TN));
-            long long blocks = p.nver << (s.nbat + (s.nm - ltm) + (s.nn - ltn));
-            kern<<<(unsigned)blocks, 256, 0, st>>>(p);
+        if constexpr (sizeof(T) == sizeof(float2)) row_roles(cn, s, p, tile_fuses(cn, si));
+        auto launch = [&](auto kern, int TM, int TN, int threads) {
+            int ltm = std::min(p.lm, __builtin_ctz(TM)), ltn = std::min(p.ln, __builtin_ctz(TN));
+            long long blocks = p.nver << (p.lbat + (p.lm - ltm) + (p.ln - ltn));
+            kern<<<(unsigned)blocks, threads, 0, st>>>(p);
         };
-        constexpr int TK = sizeof(T) == 8 ? 16 : 8;
-        switch (var) {
-            case 128064: launch(tnk::cgemm_tile<T, 128, 64, TK, 8, 4>, 128, 64); break;
-            case 64064: launch(tnk::cgemm_tile<T, 64, 64, TK, 4, 4>, 64, 64); break;
-            case 128032: launch(tnk::cgemm_tile<T, 128, 32, TK, 8, 2>, 128, 32); break;
-            case 64032: launch(tnk::cgemm_tile<T, 64, 32, TK, 4, 2>, 64, 32); break;
-            case 32032: launch(tnk::cgemm_tile<T, 32, 32, TK, 2, 2>, 32, 32); break;
-            case 128016: launch(tnk::cgemm_tile<T, 128, 16, TK, 4, 2>, 128, 16); break;
-            case 16016: launch(tnk::cgemm_tile<T, 16, 16, TK, 1, 1>, 16, 16); break;
-            default: tn_set_error("unknown kernel variant " + std::to_string(var)); return TN_EINVAL;
+        int rc = TN_OK;
+        if constexpr (sizeof(T) == sizeof(float2)) {
+            auto tile = [&](auto sw) {
+                constexpr bool SW = decltype(sw)::value;
+                switch (var) {
+                    case 128064: launch(tnk::cgemm_tile2<128, 64, 8, 8, 8, SW>, 128, 64, 128); break;
+                    case 64064: launch(tnk::cgemm_tile2<64, 64, 4, 8, 8, SW>, 64, 64, 128); break;
+                    case 128032: launch(tnk::cgemm_tile2<128, 32, 8, 4, 8, SW>, 128, 32, 128); break;
+                    case 64032: launch(tnk::cgemm_tile2<64, 32, 4, 4, 8, SW>, 64, 32, 128); break;
+                    case 32032: launch(tnk::cgemm_tile2<32, 32, 4, 2, 8, SW>, 32, 32, 128); break;
+                    case 256016: launch(tnk::cgemm_tile2<256, 16, 8, 4, 8, SW>, 256, 16, 128); break;
+                    case 128016: launch(tnk::cgemm_tile2<128, 16, 4, 4, 8, SW>, 128, 16, 128); break;
+                    case 256008: launch(tnk::cgemm_tile2<256, 8, 8, 2, 8, SW>, 256, 8, 128); break;
+                    case 256004: launch(tnk::cgemm_tile2<256, 4, 4, 2, 8, SW>, 256, 4, 128); break;
+                    case 16016: launch(tnk::cgemm_tile2<16, 16, 4, 2, 8, SW>, 16, 16, 32); break;
+                    default: rc = TN_EINVAL; break;
+                }
+            };
+            if (p.swapped) tile(std::true_type{});
+            else tile(std::false_type{});
+        } else {
+            switch (var) {
+                case 128064: launch(tnk::cgemm_tile<T, 128, 64, 8, 8, 4>, 128, 64, 256); break;
+                case 64064: launch(tnk::cgemm_tile<T, 64, 64, 8, 4, 4>, 64, 64, 256); break;
+                case 128032: launch(tnk::cgemm_tile<T, 128, 32, 8, 8, 2>, 128, 32, 256); break;
+                case 64032: launch(tnk::cgemm_tile<T, 64, 32, 8, 4, 2>, 64, 32, 256); break;
+                case 32032: launch(tnk::cgemm_tile<T, 32, 32, 8, 2, 2>, 32, 32, 256); break;
+                case 128016: launch(tnk::cgemm_tile<T, 128, 16, 8, 4, 2>, 128, 16, 256); break;
+                default: launch(tnk::cgemm_tile<T, 16, 16, 8, 1, 1>, 16, 16, 256); break;
+            }
         }
+        if (rc != TN_OK) { tn_set_error("unknown kernel variant " + std::to_string(var)); return rc; }
     }
     CK(cudaGetLastError());
     return TN_OK;
@@ -1142,7 +1184,7 @@ int launch_root_slice_sum(CNet &cn, size_t si, double2 *out, cudaStream_t st) {
     const int nfree = (int)cn.tree.nodes[root].layout.size() - nout;
     tnk::GemmParams p;
     RC(step_params(cn, cn.steps[si], p));
-    row_roles(cn, cn.steps[si], p);
+    row_roles(cn, cn.steps[si], p, row_fuses(cn, si));
     const size_t ss = cn.steps.size();
     if (cn.trace) {
         if (cn.ev_pending[ss]) {

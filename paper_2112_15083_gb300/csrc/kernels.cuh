@@ -681,6 +681,220 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN)) cgemm_tile(GemmParams p
     }
 }
 
+// Packed FP32 multiply-add: two independent fmaf in one instruction.
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long x) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(x));
+    return r;
+}
+
+// The complex64 tile kernel: products of packed FP32 pairs.  A pair is two rows of A, so the
+// four multiply-adds of a complex product take two instructions per output instead of four,
+// each with the rounding and, per output, the order of cfma (SW: with the operands exchanged,
+// as the rows hold the step's B), so the results are bit-identical to the other kernels'.
+// Bound by FP32 issue and, next to it, shared-memory reads: A sits in shared memory as planes
+// of real and imaginary parts (four rows per 16-byte read), B as complex values (two
+// columns per read, spread to pairs in registers), so an 8 x 8 thread tile reads 8 x 16
+// bytes for 256 multiply-adds.  (0, 21, 9, 7) took 28.3 ms with scalar fmaf (39 TFLOP/s),
+// 30.7 ms with packed pairs of re and im whose both orders came from shared memory, 22.5 ms so
+// (49 TFLOP/s; fmaf alone reaches 78); (15, 8, 4, 9), its operands in place, 33.1 -> 11.5 ms;
+// (11, 10, 2, 7) 4.1 -> 0.41 ms on tiles of 256 x 4.
+//
+// The longer side are the tile's rows, so a narrow step fills narrow tiles.  Each thread owns
+// groups of four adjacent rows and two adjacent columns; consecutive lanes take consecutive
+// row groups if C's lowest position is a row bit, else consecutive column groups, and
+// adjacent outputs go out in one store.  K runs in chunks of TK through two shared-memory
+// buffers; the next chunk's loads are in flight during the products.  Gathered operands
+// whose batch block is contiguous in the stored form are read in place.
+template <int TM, int TN, int RM, int RN, int TK, bool SW>
+__global__ void __launch_bounds__((TM / RM) * (TN / RN)) cgemm_tile2(GemmParams p) {
+    constexpr int NTX = TN / RN, NTY = TM / RM, NT = NTX * NTY, GM = RM / 4, GN = RN / 2;
+    constexpr int LA = (TM * TK / 2 + NT - 1) / NT, LB = (TN * TK / 2 + NT - 1) / NT;
+    static_assert(TM <= NT * LA && TN <= NT * LB, "K = 1 loads one element per slot");
+    __shared__ __align__(16) float As[2][2][TK][TM + 4];  // [buffer][re, im]
+    __shared__ __align__(16) float2 Bs[2][TK][TN + 2];
+    const int tid = threadIdx.x;
+    const bool rows_low = p.lm > 0 && p.pos_m[0] < (p.ln > 0 ? p.pos_n[0] : kMaxBits);
+    const int tx = rows_low ? tid / NTY : tid % NTX, ty = rows_low ? tid % NTY : tid / NTX;
+    const long long M = 1LL << p.lm, N = 1LL << p.ln;
+    const int lkt = min(p.lk, __ffs(TK) - 1), kt = 1 << lkt;
+    const int ltiles_m = max(0, p.lm - (__ffs(TM) - 1)), ltiles_n = max(0, p.ln - (__ffs(TN) - 1));
+    long long bid = blockIdx.x;
+    const long long n0 = (bid & ((1LL << ltiles_n) - 1)) * TN;
+    bid >>= ltiles_n;
+    const long long m0 = (bid & ((1LL << ltiles_m) - 1)) * TM;
+    bid >>= ltiles_m;
+    const long long bat = bid & ((1LL << p.lbat) - 1);
+    const long long v = bid >> p.lbat;
+    if (v >= p.nver) return;
+    const int mrows = (int)min((long long)TM, M - m0), ncols = (int)min((long long)TN, N - n0);
+    const long long eA = bat << (p.lm + p.lk), eB = bat << (p.ln + p.lk);
+    const float2 *A = (p.gA ? reinterpret_cast<const float2 *>(p.gA->src) + gather_src(*p.gA, eA, p.closed_bits)
+                            : static_cast<const float2 *>(p.ptrA[v]) + eA) + (m0 << p.lk);
+    const float2 *B = (p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, eB, p.closed_bits)
+                            : static_cast<const float2 *>(p.ptrB[v]) + eB) + (n0 << p.lk);
+    // slot i of a chunk: elements k and k + 1 of a row (K = 1: one element)
+    const int lh = max(0, lkt - 1);  // log2 slots per row
+    float4 ra[LA], rb[LB];
+    auto fetch = [&](const float2 *X, int valid, int k0, float4 *r, int n) {
+#pragma unroll
+        for (int i = 0; i < n; i++) {
+            const int s = tid + i * NT, row = s >> lh, c = (s & ((1 << lh) - 1)) << 1;
+            r[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < valid) {
+                const float2 *x = X + ((long long)row << p.lk) + k0 + c;
+                if (lkt > 0) r[i] = *reinterpret_cast<const float4 *>(x);
+                else r[i].x = x->x, r[i].y = x->y;
+            }
+        }
+    };
+    auto stage = [&](int b) {
+#pragma unroll
+        for (int i = 0; i < LA; i++) {
+            const int s = tid + i * NT, row = s >> lh, c = (s & ((1 << lh) - 1)) << 1;
+            if (row < TM) {
+                As[b][0][c][row] = ra[i].x;
+                As[b][1][c][row] = ra[i].y;
+                if (lkt > 0) {
+                    As[b][0][c + 1][row] = ra[i].z;
+                    As[b][1][c + 1][row] = ra[i].w;
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < LB; i++) {
+            const int s = tid + i * NT, row = s >> lh, c = (s & ((1 << lh) - 1)) << 1;
+            if (row < TN) {
+                Bs[b][c][row] = make_float2(rb[i].x, rb[i].y);
+                if (lkt > 0) Bs[b][c + 1][row] = make_float2(rb[i].z, rb[i].w);
+            }
+        }
+    };
+    // pair i of the thread's rows, column j: real and imaginary sums
+    unsigned long long re[RM / 2][RN], im[RM / 2][RN];
+#pragma unroll
+    for (int i = 0; i < RM / 2; i++)
+#pragma unroll
+        for (int j = 0; j < RN; j++) re[i][j] = im[i][j] = 0ull;
+    const int K = 1 << p.lk;
+    fetch(A, mrows, 0, ra, LA);
+    fetch(B, ncols, 0, rb, LB);
+    stage(0);
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = 0; k0 < K; k0 += kt, buf ^= 1) {
+        const bool more = k0 + kt < K;
+        if (more) {
+            fetch(A, mrows, k0 + kt, ra, LA);
+            fetch(B, ncols, k0 + kt, rb, LB);
+        }
+        auto mul = [&](int kk) {
+            unsigned long long ar[RM / 2], ai[RM / 2], ni[RM / 2];
+#pragma unroll
+            for (int g = 0; g < GM; g++) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&As[buf][0][kk][4 * (ty + g * NTY)]);
+                const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(&As[buf][1][kk][4 * (ty + g * NTY)]);
+                ar[2 * g] = x.x;
+                ar[2 * g + 1] = x.y;
+                ai[2 * g] = y.x;
+                ai[2 * g + 1] = y.y;
+            }
+#pragma unroll
+            for (int i = 0; i < RM / 2; i++) ni[i] = ai[i] ^ 0x8000000080000000ull;
+#pragma unroll
+            for (int h = 0; h < GN; h++) {
+                const float4 q = *reinterpret_cast<const float4 *>(&Bs[buf][kk][2 * (tx + h * NTX)]);
+#pragma unroll
+                for (int c = 0; c < 2; c++) {
+                    const int j = 2 * h + c;
+                    const unsigned long long bx = c ? pack2(q.z, q.z) : pack2(q.x, q.x);
+                    const unsigned long long by = c ? pack2(q.w, q.w) : pack2(q.y, q.y);
+#pragma unroll
+                    for (int i = 0; i < RM / 2; i++) {
+                        re[i][j] = fma2(ar[i], bx, re[i][j]);
+                        im[i][j] = SW ? fma2(ai[i], bx, im[i][j]) : fma2(ar[i], by, im[i][j]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < RM / 2; i++) {
+                        re[i][j] = fma2(ni[i], by, re[i][j]);
+                        im[i][j] = SW ? fma2(ar[i], by, im[i][j]) : fma2(ai[i], bx, im[i][j]);
+                    }
+                }
+            }
+        };
+        if (kt == TK) {
+#pragma unroll
+            for (int kk = 0; kk < TK; kk++) mul(kk);
+        } else {
+            for (int kk = 0; kk < kt; kk++) mul(kk);
+        }
+        if (more) {
+            stage(buf ^ 1);
+            __syncthreads();
+        }
+    }
+    const long long cb = scatter_bits(bat, p.pos_bat, p.lbat);
+    // adjacent outputs of a plain complex C in one store: four rows, or two columns
+    const bool row4 = p.out_fmt == OUT_C64 && p.lm >= 2 && p.pos_m[0] == 0 && p.pos_m[1] == 1;
+    const bool col2 = p.out_fmt == OUT_C64 && p.ln >= 1 && p.pos_n[0] == 0;
+    float2 *C = static_cast<float2 *>(p.C) + v * p.c_vstride;
+    const float sc = p.out_scale;
+#pragma unroll
+    for (int h = 0; h < GN; h++) {
+        const int c0 = 2 * (tx + h * NTX);
+        const long long offn0 = cb + scatter_bits(n0 + c0, p.pos_n, p.ln);
+        const long long offn1 = cb + scatter_bits(n0 + c0 + 1, p.pos_n, p.ln);
+#pragma unroll
+        for (int g = 0; g < GM; g++) {
+            const int r0 = 4 * (ty + g * NTY);
+            if (r0 >= mrows || c0 >= ncols) continue;
+            float2 x[2][4];  // column, row
+#pragma unroll
+            for (int c = 0; c < 2; c++)
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    const float2 a = unpack2(re[2 * g + i][2 * h + c]), b = unpack2(im[2 * g + i][2 * h + c]);
+                    x[c][2 * i] = make_float2(a.x, b.x);
+                    x[c][2 * i + 1] = make_float2(a.y, b.y);
+                }
+            if (row4) {
+                const long long om = scatter_bits(m0 + r0, p.pos_m, p.lm);
+#pragma unroll
+                for (int c = 0; c < 2; c++) {
+                    if (c0 + c >= ncols) break;
+                    float4 *q = reinterpret_cast<float4 *>(C + om + (c ? offn1 : offn0));
+                    q[0] = make_float4(x[c][0].x * sc, x[c][0].y * sc, x[c][1].x * sc, x[c][1].y * sc);
+                    q[1] = make_float4(x[c][2].x * sc, x[c][2].y * sc, x[c][3].x * sc, x[c][3].y * sc);
+                }
+                continue;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                if (r0 + i >= mrows) break;
+                const long long om = scatter_bits(m0 + r0 + i, p.pos_m, p.lm);
+                if (col2) {
+                    *reinterpret_cast<float4 *>(C + om + offn0) =
+                        make_float4(x[0][i].x * sc, x[0][i].y * sc, x[1][i].x * sc, x[1][i].y * sc);
+                } else {
+                    store_c(p, v, om + offn0, x[0][i]);
+                    if (c0 + 1 < ncols) store_c(p, v, om + offn1, x[1][i]);
+                }
+            }
+        }
+    }
+}
+
 // ---------------------------------------------------------------- leaves
 
 struct MatDesc {
