@@ -5,7 +5,8 @@
 // the step that consumes it, a gathered operand after its own step.  Batch-independent
 // nodes consumed by batch steps (the stem kept for later batch groups) get a reserved
 // prefix instead: batch-dependent tensors are rewritten in every group, so the two never
-// share memory.
+// share memory.  So do the results of small steps, which run out of step order (several to a
+// launch, each as soon as its operands exist): see small_step.
 #pragma once
 
 #include <algorithm>
@@ -40,9 +41,20 @@ struct CallLayout {
     std::vector<long long> nver;
     std::vector<size_t> off;
     std::vector<std::array<size_t, 2>> goff;  // per step: arena offsets of gathered operands
+    std::vector<char> small;                  // per step: result kept in the reserved prefix
     size_t arena_bytes = 0;
     double flops = 0, flops_beta = 0;
 };
+
+// Steps cheap enough to share a launch: a launch costs 2 to 4 us in a replayed graph, about
+// what 2^16 outputs over K <= 64 take on the whole chip.  Their results (at most 512 KiB
+// each, 64 MiB together) are never overwritten within an execution.
+constexpr long long kSmallOutputs = 1ll << 16, kSmallMacs = 1ll << 20;
+constexpr size_t kSmallBytes = size_t(64) << 20;
+inline bool small_step(const Step &s, long long nver) {
+    const int out = s.nbat + s.nm + s.nn;
+    return s.nk <= 6 && out <= 16 && (nver << out) <= kSmallOutputs && (nver << (out + s.nk)) <= kSmallMacs;
+}
 
 inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64_t E, int elem,
                  const std::vector<uint64_t> &slices, CallLayout &L) {
@@ -100,6 +112,17 @@ inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64
     for (const Step &s : steps)
         for (int ch : {s.a, s.b})
             if (nodes[ch].ch[0] >= 0 && !nodes[ch].beta && nodes[s.c].beta) keep[ch] = 1;
+    L.small.assign(steps.size(), 0);
+    size_t small_bytes = 0;
+    for (size_t i = 0; i < steps.size(); i++) {
+        const Step &s = steps[i];
+        if (s.c == tree.root || !small_step(s, L.nver[s.c])) continue;
+        const size_t b = (tensor_bytes(s.c) + 255) & ~size_t(255);
+        if (small_bytes + b > kSmallBytes) continue;
+        small_bytes += b;
+        L.small[i] = 1;
+        keep[s.c] = 1;
+    }
     size_t reserved = 0;
     L.off.assign(NN, 0);
     for (const Step &s : steps)

@@ -125,6 +125,12 @@ struct CallPlan {
     std::vector<tnk::GatherDesc> gd;           // batch gathers (device copy in CNet::gdescs)
     std::vector<size_t> gd_off;                // per step: first gather descriptor
     std::vector<uint64_t> gtab;                // their lookup tables (device copy in CNet::gtabs)
+    // small steps, several to a launch (tnk::small_steps): the launches of an execution with
+    // (index 0) and without (1) the batch-independent steps, in order; item i >= 0 is step i,
+    // item i < 0 small launch -1 - i, which runs blocks [small_off[-1-i], small_off[-i])
+    std::vector<char> small;                   // per step: may run in a small launch
+    std::vector<int> sched[2];
+    std::vector<size_t> small_off;
     bool valid = false;
 };
 
@@ -160,6 +166,7 @@ struct CNet {
     std::vector<int> leaf_codebits;
     std::vector<std::vector<int>> leaf_sl;  // sliced legs (e) in leg order
     DBuf arena, tables, vidx_dev, gdescs, gtabs;
+    DBuf sdescs, sblocks;  // small launches: step parameters, blocks (tnk::small_steps)
     DBuf stacks;  // stacked tensor-core tiles: the group's stack list (tnk::tc_stack_build)
     CallPlan cp;
     std::vector<int> parent;
@@ -394,6 +401,8 @@ void free_cnet(DevMem &mem, CNet &cn) {
     for (auto &b : cn.leaf_dst) release(mem, b);
     release(mem, cn.gdescs);
     release(mem, cn.gtabs);
+    release(mem, cn.sdescs);
+    release(mem, cn.sblocks);
     release(mem, cn.arena);
     release(mem, cn.tables);
     release(mem, cn.vidx_dev);
@@ -410,6 +419,8 @@ inline uint64_t leaf_code(uint64_t w, const std::vector<int> &sl) {
     for (size_t u = 0; u < sl.size(); u++) code |= ((w >> sl[u]) & 1ull) << u;
     return code;
 }
+
+int schedule_small(DevMem &mem, CNet &cn);
 
 // Versions, arena offsets and pointer tables for a slice set.
 int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, double budget) {
@@ -458,6 +469,7 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
         }
     }
     cp.off = lay.off;
+    cp.small = lay.small;
     cp.arena_bytes = lay.arena_bytes;
     if ((double)cp.arena_bytes + (double)cn.leaf_bytes > budget) {
         tn_set_error("working set of " + std::to_string(cp.arena_bytes) + " bytes exceeds the HBM budget");
@@ -634,7 +646,9 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
     cp.valid = true;
     cn.cp = std::move(cp);
     cn.variant.assign(cn.steps.size(), -1);
-    return TN_OK;
+    const int rc = schedule_small(mem, cn);
+    if (rc != TN_OK) cn.cp.valid = false;
+    return rc;
 }
 
 // Kernel variants of a step (ids as in tn_step_trace.kernel): 0 row kernel, 1 staged
@@ -1147,6 +1161,77 @@ int launch_slice_sum(CNet &cn, double2 *out, cudaStream_t st) {
     return TN_OK;
 }
 
+// The launch order with the small steps grouped: every small step whose operands exist runs in
+// the next small launch, and when none is ready the next other step follows.  The other
+// steps keep their order and a small step never runs later than its place in it, so the
+// arena's reuse (planned in step order) holds; the small steps' own results are never
+// reused.  Steps on the tensor cores, and the root (it may run fused with the slice sum), are
+// not grouped.
+int schedule_small(DevMem &mem, CNet &cn) {
+    CallPlan &cp = cn.cp;
+    const size_t ns = cn.steps.size();
+    for (size_t i = 0; i < ns; i++) {
+        const Step &s = cn.steps[i];
+        if (!cp.small[i]) continue;
+        bool ok = cn.elem == 8 && (cn.use_tc.empty() || !cn.use_tc[i]) && s.c != cn.tree.root &&
+                  cn.fmt[s.a] == tnk::OUT_C64 && cn.fmt[s.b] == tnk::OUT_C64;
+        for (size_t g = cp.gd_off[i]; g < cp.gd_off[i + 1]; g++) ok &= cp.gd[g].nver == 1 && cp.gd[g].nplanes == 1;
+        cp.small[i] = ok;
+    }
+    std::vector<tnk::GemmParams> descs;
+    std::vector<int2> blocks;
+    cp.small_off.assign(1, 0);
+    for (int skip = 0; skip < 2; skip++) {
+        std::vector<char> done(cn.tree.nodes.size(), 0);
+        std::vector<int> todo;
+        for (size_t i = 0; i < ns; i++)
+            if (!skip || cn.tree.nodes[cn.steps[i].c].beta) todo.push_back((int)i);
+        for (size_t x = 0; x < done.size(); x++) done[x] = 1;
+        for (int i : todo) done[cn.steps[i].c] = 0;
+        std::vector<int> &out = cp.sched[skip];
+        out.clear();
+        while (!todo.empty()) {
+            std::vector<int> ready, rest;
+            for (int i : todo) {
+                const Step &s = cn.steps[i];
+                (cp.small[i] && done[s.a] && done[s.b] ? ready : rest).push_back(i);
+            }
+            if (ready.size() > 1 || (ready.size() == 1 && cp.gd_off[ready[0] + 1] > cp.gd_off[ready[0]])) {
+                for (int i : ready) {
+                    const Step &s = cn.steps[i];
+                    tnk::GemmParams p;
+                    RC(step_params(cn, s, p));
+                    const auto *gd = static_cast<const tnk::GatherDesc *>(cn.gdescs.p) + cp.gd_off[i];
+                    p.gA = s.gat[0] ? gd : nullptr;
+                    p.gB = s.gat[1] ? gd + (s.gat[0] ? 1 : 0) : nullptr;
+                    const long long total = p.nver << (p.lbat + p.lm + p.ln);
+                    for (long long o = 0; o < total; o += tnk::kSmallBlock)
+                        blocks.push_back(make_int2((int)descs.size(), (int)o));
+                    descs.push_back(p);
+                }
+                out.push_back(-(int)cp.small_off.size());
+                cp.small_off.push_back(blocks.size());
+            } else if (ready.size() == 1) {
+                out.push_back(ready[0]);
+            } else {
+                ready.push_back(rest[0]);
+                out.push_back(rest[0]);
+                rest.erase(rest.begin());
+            }
+            for (int i : ready) done[cn.steps[i].c] = 1;
+            todo.swap(rest);
+        }
+    }
+    if (descs.empty()) return TN_OK;
+    RC(ensure(mem, cn.sdescs, descs.size() * sizeof(tnk::GemmParams)));
+    RC(ensure(mem, cn.sblocks, blocks.size() * sizeof(int2)));
+    CK(cudaMemcpyAsync(cn.sdescs.p, descs.data(), descs.size() * sizeof(tnk::GemmParams), cudaMemcpyHostToDevice,
+                       mem.stream));
+    CK(cudaMemcpyAsync(cn.sblocks.p, blocks.data(), blocks.size() * sizeof(int2), cudaMemcpyHostToDevice, mem.stream));
+    CK(cudaStreamSynchronize(mem.stream));
+    return TN_OK;
+}
+
 // The root step's index when it runs fused with the slice sum (-1: not fused).  Fusion
 // needs the row kernel on a root stored as plain complex values, batch, row and column
 // bits that cover the root layout once each, and free patterns that fit the fused
@@ -1210,11 +1295,26 @@ int launch_root_slice_sum(CNet &cn, size_t si, double2 *out, cudaStream_t st) {
 }
 
 // One execution of a compiled network: batch gathers, steps, FP64 slice sum into out.
+// Traced and calibrating executions, which look at each step, run the steps one by one, and
+// so do plans that prescribe each step's variant (autotune >= 2).
 int execute(CNet &cn, const uint64_t *d_closed, bool skip_beta_free, double2 *out, cudaStream_t st) {
     const long long fused = fused_root_step(cn);
-    for (const Step &s : cn.steps) {
+    const bool grouped = !cn.trace && !cn.calibrating && cn.autotune < 2 && cn.cp.valid;
+    const std::vector<int> &sched = cn.cp.sched[skip_beta_free ? 1 : 0];
+    const size_t n_items = grouped ? sched.size() : cn.steps.size();
+    for (size_t it = 0; it < n_items; it++) {
+        if (grouped && sched[it] < 0) {
+            const size_t g = (size_t)(-1 - sched[it]);
+            if (!d_closed && cn.net.n_closed > 0) { tn_set_error("execute: batch patterns missing"); return TN_EINVAL; }
+            tnk::small_steps<<<(unsigned)(cn.cp.small_off[g + 1] - cn.cp.small_off[g]), tnk::kSmallBlock, 0, st>>>(
+                static_cast<const tnk::GemmParams *>(cn.sdescs.p),
+                static_cast<const int2 *>(cn.sblocks.p) + cn.cp.small_off[g], d_closed);
+            CK(cudaGetLastError());
+            continue;
+        }
+        const size_t si = grouped ? (size_t)sched[it] : it;
+        const Step &s = cn.steps[si];
         if (skip_beta_free && !cn.tree.nodes[s.c].beta) continue;
-        const size_t si = &s - cn.steps.data();
         if ((long long)si == fused) {
             // its operands' gathers still run here unless the row kernel reads them in place
             cn.cur_closed = d_closed;

@@ -322,6 +322,59 @@ __global__ void __launch_bounds__(32 * kRowWarps) cgemm_rowstage(GemmParams p) {
     }
 }
 
+// Small steps, several to a launch: the steps of one launch have all their operands ready
+// and write disjoint results.  Block b computes outputs [blocks[b].y, blocks[b].y + 128) of
+// step descs[blocks[b].x], one per thread, accumulated as cgemm_row_one does (k ascending,
+// the step's operand order), so the bits are those of a launch of its own.  Bound by launch
+// latency: a 12-qubit circuit's 33 steps took 3.6 us each, nearly all of it the launch and
+// the wait for the step before.  Gathered operands are decoded per row if a row is
+// contiguous in the stored form, else per element.  Whole calls: that circuit 127 -> 86 us,
+// 20 qubits in split bf16 (92 steps) 501 -> 264 us.
+constexpr int kSmallBlock = 128;
+__global__ void __launch_bounds__(kSmallBlock) small_steps(const GemmParams *descs, const int2 *blocks,
+                                                           const uint64_t *closed_bits) {
+    __shared__ GemmParams p;
+    const int2 bl = blocks[blockIdx.x];
+    static_assert(sizeof(GemmParams) % 4 == 0, "copied as words");
+    for (int i = threadIdx.x; i < (int)(sizeof(GemmParams) / 4); i += kSmallBlock)
+        reinterpret_cast<uint32_t *>(&p)[i] = reinterpret_cast<const uint32_t *>(descs + bl.x)[i];
+    __syncthreads();
+    const long long o = (long long)bl.y + threadIdx.x;
+    if (o >= p.nver << (p.lbat + p.lm + p.ln)) return;
+    const long long n = o & ((1LL << p.ln) - 1), m = (o >> p.ln) & ((1LL << p.lm) - 1);
+    const long long bat = (o >> (p.ln + p.lm)) & ((1LL << p.lbat) - 1), v = o >> (p.lbat + p.lm + p.ln);
+    const int K = 1 << p.lk;
+    const long long ea = ((bat << p.lm) | m) << p.lk, eb = ((bat << p.ln) | n) << p.lk;
+    auto rows = [&](const GatherDesc *g) { return !g || (g->lb ? g->pos_beta[g->lb - 1] : g->nbits) >= p.lk; };
+    float2 acc = make_float2(0.f, 0.f);
+    if (rows(p.gA) && rows(p.gB)) {
+        const float2 *A = p.gA ? reinterpret_cast<const float2 *>(p.gA->src) + gather_src(*p.gA, ea, closed_bits)
+                               : static_cast<const float2 *>(p.ptrA[v]) + ea;
+        const float2 *B = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, eb, closed_bits)
+                               : static_cast<const float2 *>(p.ptrB[v]) + eb;
+        if (K >= 2) {
+#pragma unroll 4
+            for (int k = 0; k < K; k += 2) {
+                const float4 a = *reinterpret_cast<const float4 *>(A + k), b = *reinterpret_cast<const float4 *>(B + k);
+                acc = cfma(make_float2(a.x, a.y), make_float2(b.x, b.y), acc);
+                acc = cfma(make_float2(a.z, a.w), make_float2(b.z, b.w), acc);
+            }
+        } else {
+            acc = cfma(A[0], B[0], acc);
+        }
+    } else {
+        for (int k = 0; k < K; k++) {
+            const float2 a = p.gA ? reinterpret_cast<const float2 *>(p.gA->src)[gather_src(*p.gA, ea + k, closed_bits)]
+                                  : static_cast<const float2 *>(p.ptrA[v])[ea + k];
+            const float2 b = p.gB ? reinterpret_cast<const float2 *>(p.gB->src)[gather_src(*p.gB, eb + k, closed_bits)]
+                                  : static_cast<const float2 *>(p.ptrB[v])[eb + k];
+            acc = cfma(a, b, acc);
+        }
+    }
+    store_c(p, v, scatter_bits(bat, p.pos_bat, p.lbat) + scatter_bits(m, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln),
+            acc);
+}
+
 // mbarrier primitives (shared-memory barriers with transaction counts).
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
