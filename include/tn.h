@@ -87,11 +87,12 @@ typedef struct {
                                 (i + k - 2) mod (its variant count), so that tests can run
                                 every variant.  All variants accumulate each output over k
                                 in the same order. */
-    int32_t fuse_root_sum;   /* 1: when the root step runs the row kernel, run it fused
-                                with the FP64 slice sum (Sec. I.C step 1) in one launch
-                                whose output is bit-identical to the two launches, without
+    int32_t fuse_root_sum;   /* when the root step runs the row kernel, run it fused with
+                                the FP64 slice sum (Sec. I.C step 1) in one launch whose
+                                output is bit-identical to the two launches, without
                                 writing the root's per-slice values to memory.  0
-                                (default): separate launches. */
+                                (default): where the fused kernel's fast form applies
+                                (complex64, K <= 4); 1: always; -1: never. */
     int32_t job_groups;      /* batch groups per sampling job that the order search
                                 optimises for: a batch-independent step runs once per
                                 job, the others once per group; <= 1 (default): one */

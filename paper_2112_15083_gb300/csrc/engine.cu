@@ -152,7 +152,8 @@ struct CNet {
     const uint64_t *cur_closed = nullptr;  // batch patterns of the execution being issued
     int autotune = 1;          // 1: time the applicable variants of unseen step shapes;
                                // 0: fixed shape rules; k >= 2: variant (step + k - 2) mod count
-    bool fuse_root = false;    // run a row-kernel root step fused with the slice sum
+    int fuse_root = 0;         // run a row-kernel root step fused with the slice sum: 1 always,
+                               // 0 where the fast form applies (root_small), -1 never
     long long tc_stall = 0;    // tests only: tensor-core launches first wait this many cycles
                                // on a barrier nothing arrives on (see tn_plan_test_stall)
     DBuf err;                  // device error word of the bounded waits
@@ -1161,6 +1162,18 @@ int launch_slice_sum(CNet &cn, double2 *out, cudaStream_t st) {
     return TN_OK;
 }
 
+// Whether the root step si has the fused kernel's fast form: complex64, K of at most 4, at
+// most 2^12 free patterns (their offsets are a 32 KiB table) and operands of 32-bit
+// offsets.  Its bits equal those of the separate launches, and it is faster for every root
+// it accepts (no value of the root is written or read back), so it is on by default.
+bool root_small(const CNet &cn, size_t si) {
+    const Step &s = cn.steps[si];
+    const int nfree = (int)cn.tree.nodes[s.c].layout.size() - (int)cn.net.out_layout.size();
+    auto bits = [&](int o) { return s.gat[o] ? (int)s.g_nbits[o] : (int)cn.tree.nodes[o ? s.b : s.a].layout.size(); };
+    return cn.elem == 8 && s.nk <= 2 && nfree >= 0 && nfree <= 12 && bits(0) <= 32 && bits(1) <= 32 &&
+           cn.fmt[s.a] == tnk::OUT_C64 && cn.fmt[s.b] == tnk::OUT_C64;
+}
+
 // The launch order with the small steps grouped: every small step whose operands exist runs in
 // the next small launch, and when none is ready the next other step follows.  The other
 // steps keep their order and a small step never runs later than its place in it, so the
@@ -1238,11 +1251,11 @@ int schedule_small(DevMem &mem, CNet &cn) {
 // kernel's byte tables; it is off while FP16 scales are calibrated (every node's maximum
 // is recorded from its stored values).
 long long fused_root_step(const CNet &cn) {
-    if (!cn.fuse_root || cn.calibrating || cn.steps.empty() || !cn.cp.valid) return -1;
+    if (cn.fuse_root < 0 || cn.calibrating || cn.steps.empty() || !cn.cp.valid) return -1;
     const int root = cn.tree.root;
     const size_t si = cn.steps.size() - 1;
     const Step &s = cn.steps[si];
-    if (s.c != root) return -1;
+    if (s.c != root || (cn.fuse_root == 0 && !root_small(cn, si))) return -1;
     const int var = si < cn.variant.size() && cn.variant[si] >= 0 ? cn.variant[si] : default_variant(cn, si);
     if (var != kVarRow || cn.fmt[root] != tnk::OUT_C64) return -1;
     const int nout = (int)cn.net.out_layout.size();
@@ -1283,7 +1296,12 @@ int launch_root_slice_sum(CNet &cn, size_t si, double2 *out, cudaStream_t st) {
         CK(cudaEventRecord(cn.ev[2 * ss], st));
     }
     const unsigned blocks = (unsigned)(((1LL << nout) + 255) / 256);
-    if (cn.elem == 8) tnk::root_slice_sum<float2><<<blocks, 256, 0, st>>>(p, nfree, nout, out);
+    if (root_small(cn, si)) {
+        const size_t smem = sizeof(uint2) << nfree;
+        if (p.lk == 0) tnk::root_sum_small<0><<<blocks, 256, smem, st>>>(p, nfree, nout, out);
+        else if (p.lk == 1) tnk::root_sum_small<1><<<blocks, 256, smem, st>>>(p, nfree, nout, out);
+        else tnk::root_sum_small<2><<<blocks, 256, smem, st>>>(p, nfree, nout, out);
+    } else if (cn.elem == 8) tnk::root_slice_sum<float2><<<blocks, 256, 0, st>>>(p, nfree, nout, out);
     else tnk::root_slice_sum<double2><<<blocks, 256, 0, st>>>(p, nfree, nout, out);
     CK(cudaGetLastError());
     if (cn.trace) {
@@ -1383,6 +1401,12 @@ bool resolve_variants(CNet &cn) {
         const std::vector<int> c = step_variants(cn, si);
         if (cn.autotune >= 2 && !c.empty()) {
             cn.variant[si] = c[(si + (size_t)(cn.autotune - 2)) % c.size()];
+            continue;
+        }
+        // a root that runs fused with the slice sum (row kernel) is not timed by itself
+        if (cn.fuse_root >= 0 && cn.steps[si].c == cn.tree.root && root_small(cn, si) &&
+            std::find(c.begin(), c.end(), kVarRow) != c.end()) {
+            cn.variant[si] = kVarRow;
             continue;
         }
         // steps under ~50 us (estimated) keep the shape rules: timing them costs more
@@ -1803,7 +1827,7 @@ int tn_plan(tn_circuit_h c, const int32_t *order, int32_t n_order, const tn_edge
     p->amp.compiled = true;
     p->amp.prec = o.precision;
     p->amp.autotune = o.autotune;
-    p->amp.fuse_root = o.fuse_root_sum != 0;
+    p->amp.fuse_root = o.fuse_root_sum;
     assign_formats(p->amp);
     rc = setup_leaves(p->mem, p->amp);
     if (rc) return fail(rc);

@@ -1058,12 +1058,91 @@ __global__ void absmax_kernel(const void *data, long long n, int fmt, int *absma
 __device__ __forceinline__ double slice_widen(float x) { return tn_widen(x); }
 __device__ __forceinline__ double slice_widen(double x) { return x; }
 
+// A running FP64 sum of FP32 values with two or three FP64 additions per 16 values.
+//
+// The FP64 pipe takes 2 lanes per clock and SM, so one addition per value bounds the sum
+// (2^20 outputs of 1024 complex values: 4.1 ms, 2.1 TB/s).  Here 16 values are first added in
+// FP32 without loss, split at powers of two (emax: exponent of the largest |x|):
+// hi = (s + x) - s with s = 1.5 * 2^(emax + 4) is a multiple of 2^(emax - 19), so the 16 hi
+// parts add exactly; lo = x - hi is at most 2^(emax - 20), and the lo parts add exactly if the
+// smallest |x| is within 2^17 of the largest.  Else lo is split the same way 20 bits lower:
+// its hi parts add exactly and what is left, at most 2^(emax - 40) each, in FP32 to within
+// 2^(emax - 56), below the rounding of one FP64 addition to a sum of that size.  So 16 values
+// take at most three FP64 roundings instead of 16, and where FP64 additions one by one would
+// not round at all (most slice sums), the result is theirs.  Values FP32 cannot split
+// (infinite, NaN, or a largest one outside 2^-80 .. 2^100) are added one by one.
+// 2^14 outputs of 48 values: 16 -> 10 us; for the large sums see root_sum_small.
+struct ChunkSum {
+    double acc = 0.0;
+    __device__ __forceinline__ void one(float x) { acc = __dadd_rn(acc, slice_widen(x)); }
+    __device__ __forceinline__ void add16(const float (&x)[16]) {
+        float mx = 0.f;
+        uint32_t mn = 0xffffffffu;  // smallest 2 |bits| - 1: zeros, which add nothing, come last
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            mx = fmaxf(mx, fabsf(x[i]));
+            mn = min(mn, 2u * __float_as_uint(x[i]) - 1u);
+        }
+        if (mn == 0xffffffffu) return;  // all zero
+        // biased by 127; en is the exponent of the smallest value, or one less
+        const int ex = __float_as_int(mx) >> 23, en = (int)(mn >> 24);
+        const float s1 = __int_as_float(((ex + 4) << 23) | 0x400000);
+        float sh = 0.f, sl = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            const float hi = __fsub_rn(__fadd_rn(s1, x[i]), s1);
+            sl = __fadd_rn(sl, __fsub_rn(x[i], hi));
+            sh = __fadd_rn(sh, hi);
+        }
+        if (!(ex >= 47 && ex <= 227 && sh == sh)) {
+#pragma unroll
+            for (int i = 0; i < 16; i++) one(x[i]);
+            return;
+        }
+        if (ex - en > 17) {
+            const float s2 = __int_as_float(((ex - 16) << 23) | 0x400000);
+            float sr = 0.f;
+            sl = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+                const float lo = __fsub_rn(x[i], __fsub_rn(__fadd_rn(s1, x[i]), s1));
+                const float h2 = __fsub_rn(__fadd_rn(s2, lo), s2);
+                sl = __fadd_rn(sl, h2);
+                sr = __fadd_rn(sr, __fsub_rn(lo, h2));
+            }
+            one(sr);
+        }
+        acc = __dadd_rn(acc, __dadd_rn(slice_widen(sh), slice_widen(sl)));
+    }
+};
+
 template <typename T>
 __global__ void slice_sum(const void *const *ptr, long long nver, int nfree, int nout, double2 *out) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (1LL << nout)) return;
     double re = 0.0, im = 0.0;
     const long long nf = 1LL << nfree;
+    if constexpr (sizeof(T) == sizeof(float2)) {
+        if (nf >= 16) {
+            ChunkSum sr, si;
+            for (long long v = 0; v < nver; v++) {
+                const float2 *r = static_cast<const float2 *>(ptr[v]) + e;
+                for (long long f = 0; f < nf; f += 16) {
+                    float xr[16], xi[16];
+#pragma unroll
+                    for (int i = 0; i < 16; i++) {
+                        const float2 x = __ldcs(&r[(f + i) << nout]);
+                        xr[i] = x.x;
+                        xi[i] = x.y;
+                    }
+                    sr.add16(xr);
+                    si.add16(xi);
+                }
+            }
+            out[e] = make_double2(sr.acc, si.acc);
+            return;
+        }
+    }
     for (long long v = 0; v < nver; v++) {
         const T *r = static_cast<const T *>(ptr[v]) + e;
         long long f = 0;
@@ -1143,7 +1222,7 @@ constexpr int kRootTabBytes = 3;  // free patterns of up to 24 bits
 // The root step fused with the slice sum: out[e] = sum over explicit root versions v (in
 // order) and free patterns f (ascending) of the root product's value at C position
 // (f << nout) | e, p being the root step's row-kernel parameters.  Each value is formed
-// as the row kernel forms it and widened and added in FP64 in slice_sum's order, so out is
+// as the row kernel forms it and widened and added in FP64 as slice_sum does, so out is
 // bit-identical to the row kernel followed by slice_sum, and the root's 2^(nout + nfree)
 // values never pass through memory.  The host checks that p's batch, row and column bits
 // cover the positions [0, nout + nfree) once each, so every (bat, m, n) below is in range.
@@ -1169,23 +1248,116 @@ __global__ void __launch_bounds__(256) root_slice_sum(GemmParams p, int nfree, i
     int ne;
     root_split(p, e, be, me, ne);
     const long long nf = 1LL << nfree;
+    auto term = [&](long long v, long long f) {
+        long long bat = be, m = me;
+        int n = ne;
+        for (int j = 0; j < nbytes; j++) {
+            const int b = (int)((f >> (8 * j)) & 255);
+            bat |= tbat[j][b];
+            m |= tm[j][b];
+            n |= tn[j][b];
+        }
+        return root_scaled(p, root_value<T>(p, v, bat, m, n));
+    };
+    if constexpr (sizeof(T) == sizeof(float2)) {
+        if (nf >= 16) {
+            ChunkSum sr, si;
+            for (long long v = 0; v < p.nver; v++)
+                for (long long f = 0; f < nf; f += 16) {
+                    float xr[16], xi[16];
+#pragma unroll
+                    for (int i = 0; i < 16; i++) {
+                        const float2 x = term(v, f + i);
+                        xr[i] = x.x;
+                        xi[i] = x.y;
+                    }
+                    sr.add16(xr);
+                    si.add16(xi);
+                }
+            out[e] = make_double2(sr.acc, si.acc);
+            return;
+        }
+    }
     double re = 0.0, im = 0.0;
     for (long long v = 0; v < p.nver; v++) {
         for (long long f = 0; f < nf; f++) {
-            long long bat = be, m = me;
-            int n = ne;
-            for (int j = 0; j < nbytes; j++) {
-                const int b = (int)((f >> (8 * j)) & 255);
-                bat |= tbat[j][b];
-                m |= tm[j][b];
-                n |= tn[j][b];
-            }
-            const T x = root_scaled(p, root_value<T>(p, v, bat, m, n));
+            const T x = term(v, f);
             re = __dadd_rn(re, slice_widen(x.x));
             im = __dadd_rn(im, slice_widen(x.y));
         }
     }
     out[e] = make_double2(re, im);
+}
+
+// The same for complex64 roots with K = 2^LK of 1, 2 or 4, the fast form of the fusion.
+// Unfused, such a root writes 8 bytes per multiply-add and the slice sum reads them back:
+// (bat, m, n, k bits) = (22, 3, 5, 0) took 3.4 + 4.1 ms for 2^30 values.  Here a thread owns an
+// output and forms its terms from the operands, which are 2^-5 of the root's size and come
+// from L1.  The sliced bits of the root's position are a fixed pattern of each operand's
+// offset (they are never batch-index bits, so a gathered operand's stored block does not
+// depend on them): off[f] holds both operands' offsets of free pattern f, in elements.
+// Dynamic shared memory: 8 bytes << nfree.  The host checks the offsets fit 32 bits.
+// Now (22, 3, 5, 0) takes 1.57 ms in place of 3.4 + 4.1 ms, (20, 2, 4, 0) 0.14 in place of 0.37
+// + 0.28 ms; bound by issue (about 30 instructions per term, 16 of them the sums).
+template <int LK>
+__global__ void __launch_bounds__(256) root_sum_small(GemmParams p, int nfree, int nout, double2 *out) {
+    extern __shared__ uint2 root_off[];
+    constexpr int K = 1 << LK;
+    const int nf = 1 << nfree;
+    auto rest = [](const GatherDesc &d, long long e) {  // stored offset of e's non-batch bits
+        uint64_t r = 0;
+        for (int j = 0; j < 5; j++) r |= __ldg(&d.rest_tab[j * 256 + ((e >> (8 * j)) & 255)]);
+        return (uint32_t)r;
+    };
+    for (int f = threadIdx.x; f < nf; f += blockDim.x) {
+        long long b, m;
+        int n;
+        root_split(p, (long long)f << nout, b, m, n);
+        const long long ea = ((b << p.lm) | m) << LK, eb = ((b << p.ln) | n) << LK;
+        root_off[f] = make_uint2(p.gA ? rest(*p.gA, ea) : (uint32_t)ea, p.gB ? rest(*p.gB, eb) : (uint32_t)eb);
+    }
+    __syncthreads();
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (1LL << nout)) return;
+    long long be, me;
+    int ne;
+    root_split(p, e, be, me, ne);
+    const long long ea = ((be << p.lm) | me) << LK, eb = ((be << p.ln) | ne) << LK;
+    const long long ga = p.gA ? gather_src(*p.gA, ea, p.closed_bits) : ea;
+    const long long gb = p.gB ? gather_src(*p.gB, eb, p.closed_bits) : eb;
+    ChunkSum sr, si;
+    for (long long v = 0; v < p.nver; v++) {
+        const float2 *A = (p.gA ? reinterpret_cast<const float2 *>(p.gA->src) : static_cast<const float2 *>(p.ptrA[v])) + ga;
+        const float2 *B = (p.gB ? reinterpret_cast<const float2 *>(p.gB->src) : static_cast<const float2 *>(p.ptrB[v])) + gb;
+        auto term = [&](int f) {
+            const uint2 o = root_off[f];
+            float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const float2 a = __ldg(&A[o.x + k]), b = __ldg(&B[o.y + k]);
+                acc = p.swapped ? cfma(b, a, acc) : cfma(a, b, acc);
+            }
+            return root_scaled(p, acc);
+        };
+        int f = 0;
+        for (; f + 16 <= nf; f += 16) {
+            float xr[16], xi[16];
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+                const float2 x = term(f + i);
+                xr[i] = x.x;
+                xi[i] = x.y;
+            }
+            sr.add16(xr);
+            si.add16(xi);
+        }
+        for (; f < nf; f++) {
+            const float2 x = term(f);
+            sr.one(x.x);
+            si.one(x.y);
+        }
+    }
+    out[e] = make_double2(sr.acc, si.acc);
 }
 
 // ---------------------------------------------------------------- sampling job

@@ -277,7 +277,7 @@ class Plan:
             o.max_norm_flops = max_norm_flops
         if autotune is not None:
             o.autotune = int(autotune)
-        o.fuse_root_sum = int(bool(fuse_root_sum))
+        o.fuse_root_sum = -1 if fuse_root_sum < 0 else int(bool(fuse_root_sum))
         o.job_groups = int(job_groups)
         o.anneal_iters = int(anneal_iters)
         o.parallel_search = int(bool(parallel_search))
