@@ -405,7 +405,9 @@ typedef struct {
                        3: the root step fused with the FP64 slice sum (the root step's
                        own entry then counts no launches), 4: row kernel with rows
                        staged through shared memory, 5: long-K kernel (at most 8 x 32
-                       outputs per batch, K >= 1024), 9128 / 9064 / 9032:
+                       outputs per batch, K >= 1024), 6: row products over stacked
+                       batches (those that read the same stored block; one more launch
+                       builds the stacks), 9128 / 9064 / 9032:
                        tensor-core kernel with 128- / 64- / 32-column tiles,
                        19128 / 19064: stacked tensor-core tiles of 128 / 64 columns (the
                        batches of a group that read the same stored block of an in-place

@@ -312,6 +312,8 @@ int setup_leaves(DevMem &mem, CNet &cn) {
     if (!smem_set) {
         CK(cudaFuncSetAttribute(tnk::tc_cgemm<128, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 tnk::TcSmem<128, 3>::kBytes));
+        CK(cudaFuncSetAttribute(tnk::tc_cgemm<128, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                tnk::TcSmem<128, 3>::kBytes));
         CK(cudaFuncSetAttribute(tnk::tc_cgemm<64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 tnk::TcSmem<64, 4>::kBytes));
         CK(cudaFuncSetAttribute(tnk::tc_cgemm<32, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -422,6 +424,8 @@ inline uint64_t leaf_code(uint64_t w, const std::vector<int> &sl) {
 }
 
 int schedule_small(DevMem &mem, CNet &cn);
+bool rowstack_shape(const CNet &cn, const Step &s);
+bool skinny_fits(const CNet &cn, const Step &s);
 
 // Versions, arena offsets and pointer tables for a slice set.
 int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, double budget) {
@@ -628,9 +632,9 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
         CK(cudaMemcpyAsync(cn.gdescs.p, cp.gd.data(), cp.gd.size() * sizeof(tnk::GatherDesc), cudaMemcpyHostToDevice,
                            mem.stream));
     }
-    // the stack list of stacked tensor-core tiles (any step with an in-place A may use them)
+    // the stack list of stacked tiles and rows (any step with an in-place A may use them)
     for (size_t i = 0; i < cn.steps.size(); i++) {
-        if (!cp.tc_inplace[i][0] || cn.net.n_beta > kStackMaxBeta) continue;
+        if ((!cp.tc_inplace[i][0] && !rowstack_shape(cn, cn.steps[i])) || cn.net.n_beta > kStackMaxBeta) continue;
         RC(ensure(mem, cn.stacks, (1 + ((size_t)(tnk::kTcMaxStack + 1) << cn.net.n_beta)) * sizeof(int)));
         break;
     }
@@ -655,8 +659,9 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
 // Kernel variants of a step (ids as in tn_step_trace.kernel): 0 row kernel, 1 staged
 // small products, 4 staged row kernel, 5 long-K kernel, TM*1000+TN FFMA tile, 9128 / 9064 /
 // 9032 tensor-core tile of 128 / 64 / 32 columns, 19128 / 19064 stacked tensor-core tile of
-// 128 / 64 columns (batches sharing a stored block of A side by side).
-constexpr int kVarRow = 0, kVarSmall = 1, kVarRowStage = 4, kVarSkinny = 5, kVarTc128 = 9128, kVarTc64 = 9064,
+// 128 / 64 columns (batches sharing a stored block of A side by side), 6 row products over
+// the same stacks.
+constexpr int kVarRow = 0, kVarSmall = 1, kVarRowStage = 4, kVarSkinny = 5, kVarRowStack = 6, kVarTc128 = 9128, kVarTc64 = 9064,
               kVarTc32 = 9032, kVarTcS128 = 19128, kVarTcS64 = 19064;
 
 bool is_tc_variant(int v) {
@@ -703,6 +708,8 @@ bool small_fits(const Step &s, size_t esz) {
            (size_t)(((1 << s.nm) + (1 << s.nn)) * ((1 << s.nk) + 1)) * esz <= 48 * 1024;
 }
 
+bool rowstack_fits(const CNet &cn, size_t si);
+
 // Every variant that can run step si (the tensor-core ones when its operands are split).
 std::vector<int> step_variants(const CNet &cn, size_t si) {
     const Step &s = cn.steps[si];
@@ -718,6 +725,7 @@ std::vector<int> step_variants(const CNet &cn, size_t si) {
     }
     if (std::min(s.nm, s.nn) <= 5 && s.nk <= 6) v.push_back(kVarRow);
     if (rowstage_fits(cn, s)) v.push_back(kVarRowStage);
+    if (rowstack_fits(cn, si)) v.push_back(kVarRowStack);
     if (small_fits(s, (size_t)cn.elem)) v.push_back(kVarSmall);
     for (auto &t : kTiles)
         if (t[0] == 16 || ((2LL << std::max(s.nm, s.nn)) >= t[0] && (2LL << std::min(s.nm, s.nn)) >= t[1]))
@@ -783,6 +791,22 @@ bool tile_fuses(const CNet &cn, size_t si) {
     return true;
 }
 
+// Whether step si can run the stacked row kernel: a long side of at least 256 rows read in
+// place from a single complex version whose batch blocks are contiguous, at most 4 columns,
+// K of 4 to 16, and at most 2^14 batches per group (the stack list's limit).
+bool rowstack_shape(const CNet &cn, const Step &s) {
+    const int o = s.nn > s.nm ? 1 : 0, nb = cn.net.n_beta;
+    return cn.elem == 8 && s.gat[o] && std::max(s.nm, s.nn) >= 8 && std::min(s.nm, s.nn) <= 2 && s.nk >= 2 && s.nk <= 4 &&
+           nb >= 1 && nb <= kStackMaxBeta && s.nbat >= nb && s.nbat <= 24 && s.g_nq[o] <= 32;
+}
+bool rowstack_fits(const CNet &cn, size_t si) {
+    const Step &s = cn.steps[si];
+    if (!rowstack_shape(cn, s) || s.c == cn.tree.root || !cn.stacks.p || cn.cp.nver[s.c] != 1 || !row_fuses(cn, si)) return false;
+    const int o = s.nn > s.nm ? 1 : 0;
+    const tnk::GatherDesc &g = cn.cp.gd[cn.cp.gd_off[si] + (o == 1 && s.gat[0] ? 1 : 0)];
+    return g.pos_beta[g.lb - 1] >= s.nk + std::max(s.nm, s.nn);
+}
+
 // The long-K kernel reads a gathered operand in place when it is a single complex version
 // whose every row (K elements) is contiguous in its source.
 bool skinny_fuses(const CNet &cn, size_t si) {
@@ -799,7 +823,7 @@ bool skinny_fuses(const CNet &cn, size_t si) {
 
 // Whether variant var of step si reads its gathered operands in place (no gather launch).
 bool reads_in_place(const CNet &cn, size_t si, int var) {
-    if (var == kVarRow || var == kVarRowStage) return row_fuses(cn, si);
+    if (var == kVarRow || var == kVarRowStage || var == kVarRowStack) return row_fuses(cn, si);
     if (var == kVarSkinny) return skinny_fuses(cn, si);
     if (var >= 16000 && !is_tc_variant(var)) return tile_fuses(cn, si);
     if (is_tc_variant(var)) {
@@ -808,6 +832,25 @@ bool reads_in_place(const CNet &cn, size_t si, int var) {
         return (!s.gat[0] || cn.cp.tc_inplace[si][0]) && (!s.gat[1] || cn.cp.tc_inplace[si][1]);
     }
     return false;
+}
+
+// Operand o of step s as read in place from its stored form.
+int fill_gather(const CNet &cn, const Step &s, int o, tnk::TcGather &g) {
+    std::memset(&g, 0, sizeof(g));
+    if (!cn.cur_closed) { tn_set_error("in-place operand: batch patterns missing"); return TN_EINVAL; }
+    const int base = s.nk + (o ? s.nn : s.nm);  // read-layout position of batch bit 0
+    g.closed = cn.cur_closed;
+    g.nnb = s.nbat - cn.net.n_beta;
+    g.nq = s.g_nq[o];
+    if (s.nbat > 24 || g.nq > 32) { tn_set_error("in-place operand: gather too wide"); return TN_EUNSUPPORTED; }
+    for (int t = 0; t < cn.net.n_beta; t++) {
+        const int i = s.g_pos_beta[o][t] - base;
+        if (i < 0 || i >= s.nbat) { tn_set_error("in-place operand: beta bit outside the batch dims"); return TN_EINVAL; }
+        g.beta_mask |= 1u << i;
+        g.beta_t[i] = (int8_t)t;
+    }
+    for (int t = 0; t < g.nq; t++) g.q[t] = (int8_t)s.g_q[o][t];
+    return TN_OK;
 }
 
 template <int BN, int ST>
@@ -826,20 +869,7 @@ int launch_tc(CNet &cn, const Step &s, size_t si, const tnk::GemmParams &p, cuda
     tp.stall_cycles = cn.tc_stall;
     for (int o = 0; o < 2; o++) {
         if (cp.tc_inplace.size() <= si || !cp.tc_inplace[si][o]) continue;
-        if (!cn.cur_closed) { tn_set_error("tensor-core step: batch patterns missing"); return TN_EINVAL; }
-        tnk::TcGather &g = o ? tp.gb : tp.ga;
-        const int base = s.nk + (o ? s.nn : s.nm);  // read-layout position of batch bit 0
-        g.closed = cn.cur_closed;
-        g.nnb = s.nbat - cn.net.n_beta;
-        g.nq = s.g_nq[o];
-        if (s.nbat > 24 || g.nq > 32) { tn_set_error("tensor-core gather too wide"); return TN_EUNSUPPORTED; }
-        for (int t = 0; t < cn.net.n_beta; t++) {
-            const int i = s.g_pos_beta[o][t] - base;
-            if (i < 0 || i >= s.nbat) { tn_set_error("tensor-core gather: beta bit outside the batch dims"); return TN_EINVAL; }
-            g.beta_mask |= 1u << i;
-            g.beta_t[i] = (int8_t)t;
-        }
-        for (int t = 0; t < g.nq; t++) g.q[t] = (int8_t)s.g_q[o][t];
+        RC(fill_gather(cn, s, o, o ? tp.gb : tp.ga));
     }
     // stacked tiles: this group's stack list first (same stream), then tiles of S batches
     if (stacked) {
@@ -860,8 +890,19 @@ int launch_tc(CNet &cn, const Step &s, size_t si, const tnk::GemmParams &p, cuda
     using Lay = tnk::TcSmem<BN, ST>;
     const int fold = cp.fold.empty() ? 0 : cp.fold[si];
     const int lbn = __builtin_ctz(BN);
-    const int ltm = std::min(s.nm, 7), ltn = std::min(s.nn, lbn);
-    long long tiles_m = 1LL << (s.nm - ltm), tiles_n = 1LL << (s.nn - ltn), tiles_v = p.nver;
+    // exchange the operands where C is split and its four lowest positions are the rows' lowest
+    // bits: each lane then holds 16 adjacent outputs per plane (see tc_store16)
+    // while K is short enough for the stores to set the pace: (0, 21, 11, 7) 11.7 -> 10.3 ms,
+    // (0, 23, 7, 5) 2.7 -> 2.4 ms, but (0, 20, 8, 8) 1.13 -> 1.46 ms
+    bool swap = BN == 128 && !stacked && fold == 0 && s.nm >= 7 && s.nn >= 7 && s.nk <= 7 && p.out_fmt != tnk::OUT_C64;
+    for (int i = 0; i < 4; i++) swap = swap && s.pos_m[i] == i;
+    if (swap) {
+        std::swap(tp.lm, tp.ln);
+        std::swap(tp.ga, tp.gb);
+        for (int i = 0; i < tnk::kMaxBits; i++) std::swap(tp.pos_m[i], tp.pos_n[i]);
+    }
+    const int ltm = std::min(tp.lm, 7), ltn = std::min(tp.ln, lbn);
+    long long tiles_m = 1LL << (tp.lm - ltm), tiles_n = 1LL << (tp.ln - ltn), tiles_v = p.nver;
     if (fold == 1) { const long long vm = 128 >> s.nm; tiles_m = (p.nver + vm - 1) / vm; tiles_v = 1; }
     if (fold == 2) {
         if (s.nn > lbn) { tn_set_error("tensor-core tile narrower than a folded operand"); return TN_EINVAL; }
@@ -870,6 +911,7 @@ int launch_tc(CNet &cn, const Step &s, size_t si, const tnk::GemmParams &p, cuda
         tiles_v = 1;
     }
     const long long tiles = (tiles_m * tiles_n << s.nbat) * tiles_v;
+    if (tiles > 0x7fffffffLL - num_sms()) { tn_set_error("tensor-core step: too many tiles"); return TN_EUNSUPPORTED; }
     const long long blocks = std::min<long long>(tiles, num_sms());
     tp.C = p.C;
     tp.nver = (int)p.nver;
@@ -885,6 +927,13 @@ int launch_tc(CNet &cn, const Step &s, size_t si, const tnk::GemmParams &p, cuda
     const CUtensorMap *m = &cp.maps[cp.map_off[si]];
     // B map: box of BN rows, or of one stacked batch's N rows
     const int ib = stacked ? (s.nn == 6 ? 2 : 3) : (BN == 128 ? 1 : BN == 64 ? 2 : 3);
+    if constexpr (BN == 128) {
+        if (swap) {
+            tnk::tc_cgemm<BN, ST, true><<<(unsigned)blocks, tnk::kTcThreads, Lay::kBytes, st>>>(m[ib], m[0], tp);
+            CK(cudaGetLastError());
+            return TN_OK;
+        }
+    }
     tnk::tc_cgemm<BN, ST><<<(unsigned)blocks, tnk::kTcThreads, Lay::kBytes, st>>>(m[0], m[ib], tp);
     CK(cudaGetLastError());
     return TN_OK;
@@ -994,6 +1043,29 @@ int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
                 case 4: RC(go(tnk::cgemm_rowstage<16>)); break;
                 default: RC(go(tnk::cgemm_rowstage<32>)); break;
             }
+        }
+    } else if (var == kVarRowStack) {
+        if (!rowstack_fits(cn, si)) { tn_set_error("stacked row kernel: unsupported step shape"); return TN_EINVAL; }
+        if constexpr (sizeof(T) == sizeof(float2)) {
+            row_roles(cn, s, p, true);
+            tnk::TcGather g;
+            RC(fill_gather(cn, s, s.nn > s.nm ? 1 : 0, g));
+            const int S = tnk::kTcMaxStack;
+            int *stack = static_cast<int *>(cn.stacks.p);
+            tnk::tc_stack_build<<<1, 1024, (size_t)8 << cn.net.n_beta, st>>>(g, cn.net.n_beta, S, stack);
+            CK(cudaGetLastError());
+            // items of up to 2048 rows; the number of stacks is known on the device only
+            const long long most = (1LL << (s.nbat + p.lm - 8));
+            const unsigned blocks = (unsigned)std::min<long long>(most, 4LL * num_sms());
+            auto by_k = [&](auto n_tag) {
+                constexpr int N = decltype(n_tag)::value;
+                if (p.lk == 2) tnk::cgemm_rowstack<N, 4><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
+                else if (p.lk == 3) tnk::cgemm_rowstack<N, 8><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
+                else tnk::cgemm_rowstack<N, 16><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
+            };
+            if (p.ln == 0) by_k(std::integral_constant<int, 1>{});
+            else if (p.ln == 1) by_k(std::integral_constant<int, 2>{});
+            else by_k(std::integral_constant<int, 4>{});
         }
     } else if (var == kVarSkinny) {
         if (!skinny_fits(cn, s)) { tn_set_error("long-K kernel: unsupported step shape"); return TN_EINVAL; }
@@ -1387,7 +1459,7 @@ std::vector<long long> tune_key(const CNet &cn, size_t si) {
     const bool ipa = cn.cp.tc_inplace.size() > si && cn.cp.tc_inplace[si][0];
     const bool ipb = cn.cp.tc_inplace.size() > si && cn.cp.tc_inplace[si][1];
     return {cn.elem, cn.use_tc.empty() ? 0 : cn.use_tc[si], cn.cp.fold.empty() ? 0 : cn.cp.fold[si], cn.fmt[s.a],
-            cn.fmt[s.c], s.nbat, s.nm, s.nn, s.nk, cn.cp.nver[s.c], ipa + 2 * ipb + 4 * stack_fits(cn, si, 128)};
+            cn.fmt[s.c], s.nbat, s.nm, s.nn, s.nk, cn.cp.nver[s.c], ipa + 2 * ipb + 4 * stack_fits(cn, si, 128) + 8 * rowstack_fits(cn, si) + 16 * tile_fuses(cn, si)};
 }
 
 // Fill in every step's variant that is known (single candidate, autotuning off, or a

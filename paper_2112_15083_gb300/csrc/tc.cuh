@@ -91,21 +91,22 @@ __global__ void __launch_bounds__(1024) tc_stack_build(TcGather g, int nbeta, in
         keys[b] = ((unsigned long long)(unsigned)tc_gather_sel(g, g.closed[b]) << 32) | (unsigned)b;
     for (int i = tid; i < T * (S + 1); i += nt) out[1 + i] = -1;
     __syncthreads();
+    // a thread owns pair t of a stage, so stages with j <= 32 stay inside a warp's 64 keys
     for (int k = 2; k <= T; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = tid; i < T; i += nt) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const unsigned long long a = keys[i], c = keys[l];
-                    if ((a > c) == ((i & k) == 0)) {
-                        keys[i] = c;
-                        keys[l] = a;
-                    }
+            for (int t = tid; t < T / 2; t += nt) {
+                const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), l = i | j;
+                const unsigned long long x = keys[i], y = keys[l];
+                if ((x > y) == ((i & k) == 0)) {
+                    keys[i] = y;
+                    keys[l] = x;
                 }
             }
-            __syncthreads();
+            if (j > 32 || (j == 1 && k > 32)) __syncthreads();
+            else __syncwarp();
         }
     }
+    __syncthreads();
     // thread tid walks positions [lo, hi) of the sorted list; a run starts where the block
     // changes, and a stack at every S-th position of a run
     const int E = (T + nt - 1) / nt, lo = min(T, tid * E), hi = min(T, lo + E);
@@ -152,6 +153,97 @@ __global__ void __launch_bounds__(1024) tc_stack_build(TcGather g, int nbeta, in
     if (tid == nt - 1) out[0] = scan[tid];
 }
 
+// Row products over the stack list: C[bat][m][n] = sum_k A[bat][m][k] B[bat][n][k] for a long
+// row side read in place from stored blocks, N <= 4 columns and K <= 16.  The row kernel reads
+// every batch's block anew (16384 batches of 1 MB each from 4096 stored blocks: 17 GB through
+// L1, 16 bytes of 32 rows per instruction; (bat, m, n, k bits) = (14, 13, 0, 4) took 5.4 ms);
+// here a block of threads takes up to 2048 rows of a stored block, 256 at a time, each thread
+// one row in registers (staged through padded shared memory with coalesced loads), and
+// applies them to the stack's batches; the addresses are decoded once per 2048 rows.  Each output's products and order are the row kernel's.  The same step: 5.4 -> 1.46 ms
+// (3.1 ms with an item per 256 rows, whose decode then took as long as its rows).
+constexpr int kRowStackRows = 256, kRowStackChunks = 8;  // rows per pass, passes per item
+template <int N, int K>
+__global__ void __launch_bounds__(kRowStackRows) cgemm_rowstack(GemmParams p, TcGather g, const int *stack, int S) {
+    constexpr int kPitch = 8 * K + 16;  // bytes between staged rows: 16-byte reads without conflicts
+    __shared__ __align__(16) unsigned char stage[kRowStackRows * kPitch];
+    __shared__ __align__(16) float2 vec[kTcMaxStack][N * K];
+    __shared__ long long cbase[kTcMaxStack];
+    __shared__ const float2 *src[1 + kTcMaxStack];  // the block, the batches' columns
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int passes = min(kRowStackChunks, 1 << (p.lm - 8)), groups = (1 << (p.lm - 8)) / passes;
+    const long long items = (long long)stack[0] * groups << g.nnb;
+    unsigned char *mine = stage + warp * 32 * kPitch;
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+        const long long q = it / groups;
+        const int row0 = (int)(it - q * groups) * passes * kRowStackRows, nonb = (int)(q & ((1 << g.nnb) - 1));
+        const int *e = stack + 1 + (q >> g.nnb) * (S + 1);
+        __syncthreads();  // the shared words of the previous item
+        // one thread per address: the block's, then the batches'
+        if (tid <= S) {
+            const int beta = e[max(1, tid)];
+            src[tid] = nullptr;
+            if (beta >= 0) {
+                const long long bat = tc_compose_bat(g, p.lbat, nonb, beta);
+                if (tid == 0) {
+                    src[0] = reinterpret_cast<const float2 *>(p.gA->src) +
+                             gather_src(*p.gA, bat << (p.lm + p.lk), p.closed_bits);
+                } else {
+                    const long long eb = bat << (p.ln + p.lk);
+                    src[tid] = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, eb, p.closed_bits)
+                                    : static_cast<const float2 *>(p.ptrB[0]) + eb;
+                    cbase[tid - 1] = scatter_bits(bat, p.pos_bat, p.lbat);
+                }
+            }
+        }
+        __syncthreads();
+        // the warp's 32 rows of a pass: 16 K float4, consecutive lanes consecutive addresses
+        const float4 *A = reinterpret_cast<const float4 *>(src[0] + ((long long)(row0 + warp * 32) << p.lk)) + lane;
+        float4 in[K / 2];
+#pragma unroll
+        for (int i = 0; i < K / 2; i++) in[i] = __ldg(A + i * 32);
+        int cnt = 0;
+        while (cnt < S && src[1 + cnt]) cnt++;
+        for (int i = tid; i < cnt * N * K; i += kRowStackRows) vec[i / (N * K)][i % (N * K)] = __ldg(src[1 + i / (N * K)] + i % (N * K));
+        __syncthreads();
+        for (int c = 0; c < passes; c++) {
+#pragma unroll
+            for (int i = 0; i < K / 2; i++) {
+                const int o = i * 32 + lane;
+                *reinterpret_cast<float4 *>(mine + (o / (K / 2)) * kPitch + 16 * (o % (K / 2))) = in[i];
+            }
+            __syncwarp();
+            float2 a[K];
+#pragma unroll
+            for (int i = 0; i < K / 2; i++) {
+                const float4 x = *reinterpret_cast<const float4 *>(mine + lane * kPitch + 16 * i);
+                a[2 * i] = make_float2(x.x, x.y);
+                a[2 * i + 1] = make_float2(x.z, x.w);
+            }
+            __syncwarp();
+            if (c + 1 < passes) {  // the next pass's rows are in flight during this one's products
+                A += kRowStackRows * K / 2;
+#pragma unroll
+                for (int i = 0; i < K / 2; i++) in[i] = __ldg(A + i * 32);
+            }
+            const long long offm = scatter_bits(row0 + c * kRowStackRows + tid, p.pos_m, p.lm);
+            for (int j = 0; j < cnt; j++) {
+#pragma unroll
+                for (int n = 0; n < N; n++) {
+                    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < K / 2; i++) {
+                        const float4 y = *reinterpret_cast<const float4 *>(&vec[j][n * K + 2 * i]);
+                        const float2 y0 = make_float2(y.x, y.y), y1 = make_float2(y.z, y.w);
+                        acc = p.swapped ? cfma(y0, a[2 * i], acc) : cfma(a[2 * i], y0, acc);
+                        acc = p.swapped ? cfma(y1, a[2 * i + 1], acc) : cfma(a[2 * i + 1], y1, acc);
+                    }
+                    store_c(p, 0, cbase[j] + offm + scatter_bits(n, p.pos_n, p.ln), acc);
+                }
+            }
+        }
+    }
+}
+
 struct TcParams {
     void *C;                 // output base (version 0); version v at C + 8 * v * c_plane bytes
     long long c_plane;       // elements per version (= split plane stride)
@@ -178,37 +270,40 @@ struct TcParams {
 // the plain n-fastest order).
 struct TcTile {
     int tn_i, tm_i, bat;
-    long long v;
+    int v;
 };
 
 // Stacked tile t: m tiles fastest, then stacks (sorted by block: the stacks of one block
 // run back to back and share its panels in L2), then the non-beta batch bits, then version.
+// Tile counts fit 32 bits (the host checks), which keeps the divisions short: the producer
+// forms them between copies.
 struct TcStackTile {
     int tm_i, stack, nonb;
-    long long v;
+    int v;
 };
-__device__ __forceinline__ TcStackTile tc_stack_tile(long long t, long long tiles_m, int n_stacks, int nnb) {
+__device__ __forceinline__ TcStackTile tc_stack_tile(uint32_t t, uint32_t tiles_m, uint32_t n_stacks, int nnb) {
     TcStackTile r;
-    r.tm_i = (int)(t % tiles_m);
-    long long q = t / tiles_m;
-    r.stack = (int)(q % n_stacks);
-    q /= n_stacks;
-    r.nonb = (int)(q & ((1LL << nnb) - 1));
-    r.v = q >> nnb;
+    uint32_t q = t / tiles_m;
+    r.tm_i = (int)(t - q * tiles_m);
+    const uint32_t z = q / n_stacks;
+    r.stack = (int)(q - z * n_stacks);
+    r.nonb = (int)(z & ((1u << nnb) - 1));
+    r.v = (int)(z >> nnb);
     return r;
 }
 
-__device__ __forceinline__ TcTile tc_tile(long long t, long long tiles_m, long long tiles_n, int lbat, int group_m) {
-    const long long per_bat = tiles_m * tiles_n;
-    const long long bv = t / per_bat, tl = t - bv * per_bat;
+__device__ __forceinline__ TcTile tc_tile(uint32_t t, uint32_t tiles_m, uint32_t tiles_n, int lbat, uint32_t group_m) {
+    const uint32_t per_bat = tiles_m * tiles_n;
+    const uint32_t bv = t / per_bat, tl = t - bv * per_bat;
     TcTile r;
-    r.bat = (int)(bv & ((1LL << lbat) - 1));
-    r.v = bv >> lbat;
-    const long long gsz = (long long)group_m * tiles_n;
-    const long long g = tl / gsz, rr = tl - g * gsz;
-    const long long gm = min((long long)group_m, tiles_m - g * group_m);
-    r.tn_i = (int)(rr / gm);
-    r.tm_i = (int)(g * group_m + rr % gm);
+    r.bat = (int)(bv & ((1u << lbat) - 1));
+    r.v = (int)(bv >> lbat);
+    const uint32_t gsz = group_m * tiles_n;
+    const uint32_t g = tl / gsz, rr = tl - g * gsz;
+    const uint32_t gm = min(group_m, tiles_m - g * group_m);
+    const uint32_t n = rr / gm;
+    r.tn_i = (int)n;
+    r.tm_i = (int)(g * group_m + rr - n * gm);
     return r;
 }
 
@@ -414,7 +509,11 @@ constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;  // warp 0: TMA, warp 1: MMA, 
 // the A row panel).  Operand maps are 4-D: [version][4 * BAT planes][rows][K].
 // TMEM holds two accumulator pairs (Cr | Ci for BN columns each) so the epilogue of
 // one tile overlaps the MMAs of the next.
-template <int BN, int STAGES>
+// SW: the operands are exchanged (A holds the step's B, p.vidx's halves as for the step): the
+// planes of each product swap sides and the products keep their order, so the bits are the
+// same.  The engine exchanges them where C is split with m lowest, which puts 16 adjacent
+// outputs into one lane (its rule, with both sides measured, stands at the launch).
+template <int BN, int STAGES, bool SW = false>
 __global__ void __launch_bounds__(kTcThreads, 1)
     tc_cgemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcParams p) {
     using L = TcSmem<BN, STAGES>;
@@ -437,15 +536,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int ltm = min(p.lm, 7), ltn = min(p.ln, __ffs(BN) - 1);
     const int vm = p.fold == 1 ? (kTcBM >> p.lm) : 1;  // versions per m tile
     const int vn = p.fold == 2 ? (BN >> p.ln) : 1;      // versions per n tile
-    const long long tiles_m = p.fold == 1 ? (p.nver + vm - 1) / vm : (1LL << (p.lm - ltm));
-    const long long tiles_n = p.fold == 2 ? (p.nver + vn - 1) / vn : (1LL << (p.ln - ltn));
-    const long long tiles_v = p.fold ? 1 : p.nver;
-    const long long per_bat = tiles_m * tiles_n;
+    const uint32_t tiles_m = p.fold == 1 ? (p.nver + vm - 1) / vm : (1u << (p.lm - ltm));
+    const uint32_t tiles_n = p.fold == 2 ? (p.nver + vn - 1) / vn : (1u << (p.ln - ltn));
+    const uint32_t tiles_v = p.fold ? 1 : p.nver;
     // stacked: (version, non-beta bits, stack, m tile); the host guarantees one n tile
     const bool stk = p.stack != nullptr;
     const int S = p.stack_S, n_stacks = stk ? p.stack[0] : 0;
-    const long long ntiles =
-        stk ? tiles_m * n_stacks * (1LL << p.ga.nnb) * tiles_v : per_bat * (1LL << p.lbat) * tiles_v;
+    const uint32_t ntiles = (stk ? (tiles_m * n_stacks << p.ga.nnb) : (tiles_m * tiles_n << p.lbat)) * tiles_v;
     const int BAT = 1 << p.lbat;
     const int K = 1 << p.lk;
     const int nkb = (K + kTcBK - 1) / kTcBK;
@@ -479,24 +576,24 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
     long long issued = 0;  // producer: ring slots issued
     if (warp == 0) {
-        if (lane == 0) {
-            long long slot = 0;
-            bool ok = true;
-            for (long long t = blockIdx.x; t < ntiles && ok && !stk; t += gridDim.x) {
+        const int sza = p.ga.closed ? 1 << (p.ga.nnb + p.ga.nq) : BAT;
+        const int szb = p.gb.closed ? 1 << (p.gb.nnb + p.gb.nq) : BAT;
+        int s = 0;
+        uint32_t par = 1;  // of the empty barrier the next slot waits for
+        bool ok = true;
+        if (!stk && lane == 0) {
+            for (uint32_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
                 const TcTile tt = tc_tile(t, tiles_m, tiles_n, p.lbat, p.group_m);
-                const int tn_i = tt.tn_i, tm_i = tt.tm_i, bat = tt.bat, v = (int)tt.v;
-                const int ia = p.fold == 1 ? p.vidx[0] + tm_i * vm : p.vidx[p.fold == 2 ? 0 : v];
-                const int ib = p.fold == 2 ? p.vidx[p.nver] + tn_i * vn : p.vidx[p.nver + (p.fold == 1 ? 0 : v)];
+                const int tn_i = tt.tn_i, tm_i = tt.tm_i, bat = tt.bat, v = tt.v;
+                const int *va = p.vidx + (SW ? p.nver : 0), *vb = p.vidx + (SW ? 0 : p.nver);
+                const int ia = p.fold == 1 ? va[0] + tm_i * vm : va[p.fold == 2 ? 0 : v];
+                const int ib = p.fold == 2 ? vb[0] + tn_i * vn : vb[p.fold == 1 ? 0 : v];
                 const int rowA = p.fold == 1 ? 0 : tm_i * kTcBM, rowB = p.fold == 2 ? 0 : tn_i * BN;
                 // plane coordinates: plane pl of batch bat, or of its stored pattern block
                 const int pza = p.ga.closed ? tc_gather_plane(p.ga, p.lbat, bat) : bat;
                 const int pzb = p.gb.closed ? tc_gather_plane(p.gb, p.lbat, bat) : bat;
-                const int sza = p.ga.closed ? 1 << (p.ga.nnb + p.ga.nq) : BAT;
-                const int szb = p.gb.closed ? 1 << (p.gb.nnb + p.gb.nq) : BAT;
-                for (int kb = 0; kb < nkb; kb++, slot++) {
-                    const int s = (int)(slot % STAGES);
-                    if (slot >= STAGES &&
-                        !mbar_wait(smem_u32(&empty[s]), (uint32_t)(((slot / STAGES) & 1) ^ 1), abort_flag, kLimit)) {
+                for (int kb = 0; kb < nkb; kb++) {
+                    if (issued >= STAGES && !mbar_wait(smem_u32(&empty[s]), par, abort_flag, kLimit)) {
                         ok = false;
                         break;
                     }
@@ -508,76 +605,84 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         tma_load_4d(smem_u32(st + 4 * L::kAPlane + pl * L::kBPlane), &tmB, kb * kTcBK, rowB,
                                     pl * szb + pzb, ib, fb);
                     }
-                    issued = slot + 1;
+                    issued++;
+                    if (++s == STAGES) {
+                        s = 0;
+                        par ^= 1u;
+                    }
                 }
             }
-            // stacked tiles: one A panel, then one (1 << ln)-row B box per batch of the stack
-            // (its valid slots come first); the next tile's stack entry is loaded while this
-            // tile's slots are issued, and every slot tells the MMA thread its width
-            auto entry = [&](long long t) {
-                return p.stack + 1 + (long long)tc_stack_tile(t, tiles_m, n_stacks, p.ga.nnb).stack * (S + 1);
-            };
-            int nx[kTcMaxStack + 1];
-            if (stk && blockIdx.x < ntiles) {
-                const int *sb = entry(blockIdx.x);
-#pragma unroll
-                for (int j = 0; j <= kTcMaxStack; j++) nx[j] = j <= S ? sb[j] : -1;
+        }
+        // Stacked tiles: one A panel, then one (1 << ln)-row B box per batch of the stack (its
+        // valid slots come first); every slot tells the MMA thread its width.  Decoding a tile
+        // takes a chain of loads (stack entry, batch patterns) and divisions as long as several
+        // ring slots, so the warp decodes the next tile, one lane per batch, right after it has
+        // issued the first slot of this one, while the ring is full: (12, 11, 5, 8) 1.95 ->
+        // 1.80 ms.  (The same for unstacked tiles, whose decode is short, made them 10% slower.)
+        struct Dec {
+            int pza, pzb, rowA, ia, ib, nbox;
+        };
+        auto decode = [&](uint32_t t) {
+            Dec d;
+            const TcStackTile tt = tc_stack_tile(t, tiles_m, n_stacks, p.ga.nnb);
+            const int *e = p.stack + 1 + (long long)tt.stack * (S + 1);
+            const int beta = lane < S ? e[1 + lane] : -1;
+            d.pza = tt.nonb | (e[0] << p.ga.nnb);  // the block the stack selects
+            d.pzb = 0;
+            if (beta >= 0) {
+                const int bat = tc_compose_bat(p.ga, p.lbat, tt.nonb, beta);
+                d.pzb = p.gb.closed ? tc_gather_plane(p.gb, p.lbat, bat) : bat;
             }
-            for (long long t = blockIdx.x; t < ntiles && ok && stk; t += gridDim.x) {
-                int e[kTcMaxStack + 1];
+            d.nbox = __popc(__ballot_sync(0xffffffffu, beta >= 0));
+            d.rowA = tt.tm_i * kTcBM;
+            d.ia = p.vidx[tt.v];
+            d.ib = p.vidx[p.nver + tt.v];
+            return d;
+        };
+        const int bbox = (kTcBK * 2) << p.ln;  // bytes per B box
+        Dec next = {0, 0, 0, 0, 0, 0};
+        if (stk && blockIdx.x < ntiles) next = decode(blockIdx.x);
+        for (uint32_t t = blockIdx.x; t < ntiles && ok && stk; t += gridDim.x) {
+            const Dec d = next;
+            int pzb[kTcMaxStack];
 #pragma unroll
-                for (int j = 0; j <= kTcMaxStack; j++) e[j] = nx[j];
-                if (t + gridDim.x < ntiles) {
-                    const int *sb = entry(t + gridDim.x);
+            for (int j = 0; j < kTcMaxStack; j++) pzb[j] = __shfl_sync(0xffffffffu, d.pzb, j);
+            for (int kb = 0; kb < nkb; kb++) {
+                if (lane == 0) {
+                    if (issued >= STAGES) ok = mbar_wait(smem_u32(&empty[s]), par, abort_flag, kLimit);
+                    if (ok) {
+                        slot_cols[s] = d.nbox << p.ln;  // published by the arrive below
+                        const uint32_t fb = smem_u32(&full[s]);
+                        mbar_expect_tx(fb, (uint32_t)(4 * L::kAPlane + 4 * d.nbox * bbox));
+                        unsigned char *st = smem + s * L::kStage;
 #pragma unroll
-                    for (int j = 0; j <= kTcMaxStack; j++) nx[j] = j <= S ? sb[j] : -1;
-                }
-                const TcStackTile tt = tc_stack_tile(t, tiles_m, n_stacks, p.ga.nnb);
-                const int pza = tt.nonb | (e[0] << p.ga.nnb);  // the block the stack selects
-                const int sza = 1 << (p.ga.nnb + p.ga.nq);
-                int pzb[kTcMaxStack], nbox = 0;
+                        for (int pl = 0; pl < 4; pl++) {
+                            tma_load_4d(smem_u32(st + pl * L::kAPlane), &tmA, kb * kTcBK, d.rowA, pl * sza + d.pza, d.ia, fb);
 #pragma unroll
-                for (int j = 0; j < kTcMaxStack; j++) {
-                    pzb[j] = -1;
-                    if (e[1 + j] >= 0) {
-                        const int bat = tc_compose_bat(p.ga, p.lbat, tt.nonb, e[1 + j]);
-                        pzb[j] = p.gb.closed ? tc_gather_plane(p.gb, p.lbat, bat) : bat;
-                        nbox++;
+                            for (int j = 0; j < kTcMaxStack; j++)
+                                if (j < d.nbox)
+                                    tma_load_4d(smem_u32(st + 4 * L::kAPlane + pl * L::kBPlane + j * bbox), &tmB,
+                                                kb * kTcBK, 0, pl * szb + pzb[j], d.ib, fb);
+                        }
                     }
                 }
-                const int ia = p.vidx[tt.v], ib = p.vidx[p.nver + tt.v];
-                const int rowA = tt.tm_i * kTcBM;
-                const int szb = p.gb.closed ? 1 << (p.gb.nnb + p.gb.nq) : BAT;
-                const int bbox = (kTcBK * 2) << p.ln;  // bytes per B box
-                for (int kb = 0; kb < nkb; kb++, slot++) {
-                    const int s = (int)(slot % STAGES);
-                    if (slot >= STAGES &&
-                        !mbar_wait(smem_u32(&empty[s]), (uint32_t)(((slot / STAGES) & 1) ^ 1), abort_flag, kLimit)) {
-                        ok = false;
-                        break;
-                    }
-                    slot_cols[s] = nbox << p.ln;  // published by the arrive below
-                    const uint32_t fb = smem_u32(&full[s]);
-                    mbar_expect_tx(fb, (uint32_t)(4 * L::kAPlane + 4 * nbox * bbox));
-                    unsigned char *st = smem + s * L::kStage;
-                    for (int pl = 0; pl < 4; pl++) {
-                        tma_load_4d(smem_u32(st + pl * L::kAPlane), &tmA, kb * kTcBK, rowA, pl * sza + pza, ia, fb);
-#pragma unroll
-                        for (int j = 0; j < kTcMaxStack; j++)
-                            if (pzb[j] >= 0)
-                                tma_load_4d(smem_u32(st + 4 * L::kAPlane + pl * L::kBPlane + j * bbox), &tmB,
-                                            kb * kTcBK, 0, pl * szb + pzb[j], ib, fb);
-                    }
-                    issued = slot + 1;
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                if (!ok) break;
+                issued++;
+                if (++s == STAGES) {
+                    s = 0;
+                    par ^= 1u;
                 }
+                if (kb == 0 && t + gridDim.x < ntiles) next = decode(t + gridDim.x);
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             // products (A plane, B plane, accumulator 0 = Cr / 1 = Ci, negate A);
             // planes: 0 re_hi, 1 re_lo, 2 im_hi, 3 im_lo
-            const int8_t pa[12] = {0, 0, 1, 2, 2, 3, 0, 0, 1, 2, 2, 3};
-            const int8_t pb[12] = {0, 1, 0, 2, 3, 2, 2, 3, 2, 0, 1, 0};
+            const int8_t p0[12] = {0, 0, 1, 2, 2, 3, 0, 0, 1, 2, 2, 3};
+            const int8_t p1[12] = {0, 1, 0, 2, 3, 2, 2, 3, 2, 0, 1, 0};
+            const int8_t(&pa)[12] = SW ? p1 : p0, (&pb)[12] = SW ? p0 : p1;
             const int8_t acc[12] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1};
             const int8_t neg[12] = {0, 0, 0, 1, 1, 1, 0, 0, 0, 0, 0, 0};
             uint32_t id_pos = idesc_f16(BN, p.in_fp16, false), id_neg = idesc_f16(BN, p.in_fp16, true);
@@ -587,7 +692,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             bool ok = true;
             // test hook: a wait that runs out before any MMA is issued
             if (p.stall_cycles > 0) ok = mbar_wait(smem_u32(never), 0u, abort_flag, p.stall_cycles);
-            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, it++) {
+            for (uint32_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, it++) {
                 const int b = it & 1;
                 if (it >= 2 &&
                     !mbar_wait(smem_u32(&acc_empty[b]), (uint32_t)(((it >> 1) & 1) ^ 1), abort_flag, kLimit)) {

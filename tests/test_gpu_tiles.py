@@ -42,3 +42,29 @@ def test_every_variant_gives_the_same_bits(case):
         assert np.array_equal(got, ref), (case, r)
     if rows * cols == 24:
         assert {128064, 64064, 128032, 64032, 32032, 256016, 128016, 256008, 256004, 16016} <= seen, sorted(seen)
+
+
+# steps with a short side of up to 4 and K <= 16 whose long operand is read in place: the row
+# kernels and the row products over stacked batches (kernel 6); ragged last groups
+@pytest.mark.parametrize("case", [(4, 5, 11, 6, 8), (4, 5, 11, 6, 9), (4, 6, 8, 8, 8)])
+def test_stacked_rows_give_the_same_bits(case):
+    import paper_2112_15083_gb300 as P
+    rows, cols, cycles, sliced, lb = case
+    C = P.circuit_load(cg.sycamore_grid(rows, cols, cycles, seed=0).serialize())
+    openq = cg.default_open_qubits(rows, cols, 6)
+    cb = cg.random_closed_bits((1 << lb) + 77, rows * cols - 6, seed=9)
+    cb[5:40] = cb[4]  # more batches on one stored block than a stack holds
+    kw = dict(n_auto_sliced=sliced, log2_batches=lb, order_trials=16)
+    plan = P.plan(C, openq, autotune=0, **kw)
+    sl = np.arange(1 << len(plan.sliced_edges()), dtype=np.uint64)
+    ref = plan.contract(sl, cb)
+    seen = set()
+    for r in range(6):
+        p = P.plan(C, openq, autotune=2 + r, **kw)
+        p.trace(True)
+        got = p.contract(sl, cb)
+        seen |= {s["kernel"] for s in p.trace_read() if s["launches"]}
+        p.trace(False)
+        assert np.array_equal(got, ref), (case, r)
+    if lb == 8:
+        assert 6 in seen, sorted(seen)
