@@ -47,13 +47,13 @@ struct CallLayout {
 };
 
 // Steps cheap enough to share a launch: a launch costs 2 to 4 us in a replayed graph, about
-// what 2^16 outputs over K <= 64 take on the whole chip.  Their results (at most 512 KiB
+// what 2^18 outputs over a short K take on the whole chip.  Their results (at most 2 MiB
 // each, 64 MiB together) are never overwritten within an execution.
-constexpr long long kSmallOutputs = 1ll << 16, kSmallMacs = 1ll << 20;
+constexpr long long kSmallOutputs = 1ll << 18, kSmallMacs = 1ll << 21, kSmallAlone = 1ll << 15;
 constexpr size_t kSmallBytes = size_t(64) << 20;
 inline bool small_step(const Step &s, long long nver) {
     const int out = s.nbat + s.nm + s.nn;
-    return s.nk <= 6 && out <= 16 && (nver << out) <= kSmallOutputs && (nver << (out + s.nk)) <= kSmallMacs;
+    return s.nk <= 6 && out <= 18 && (nver << out) <= kSmallOutputs && (nver << (out + s.nk)) <= kSmallMacs;
 }
 
 inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64_t E, int elem,

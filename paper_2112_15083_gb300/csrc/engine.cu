@@ -127,10 +127,12 @@ struct CallPlan {
     std::vector<uint64_t> gtab;                // their lookup tables (device copy in CNet::gtabs)
     // small steps, several to a launch (tnk::small_steps): the launches of an execution with
     // (index 0) and without (1) the batch-independent steps, in order; item i >= 0 is step i,
-    // item i < 0 small launch -1 - i, which runs blocks [small_off[-1-i], small_off[-i])
+    // item i < 0 launches levels small_run[-1 - i] = {first, count}; level l is the blocks
+    // [small_off[l], small_off[l + 1])
     std::vector<char> small;                   // per step: may run in a small launch
     std::vector<int> sched[2];
-    std::vector<size_t> small_off;
+    std::vector<int> small_off;
+    std::vector<std::array<int, 2>> small_run;
     bool valid = false;
 };
 
@@ -167,7 +169,7 @@ struct CNet {
     std::vector<int> leaf_codebits;
     std::vector<std::vector<int>> leaf_sl;  // sliced legs (e) in leg order
     DBuf arena, tables, vidx_dev, gdescs, gtabs;
-    DBuf sdescs, sblocks;  // small launches: step parameters, blocks (tnk::small_steps)
+    DBuf sdescs, sblocks, slevels;  // small launches: step parameters, blocks, small_off (tnk::small_steps)
     DBuf stacks;  // stacked tensor-core tiles: the group's stack list (tnk::tc_stack_build)
     CallPlan cp;
     std::vector<int> parent;
@@ -406,6 +408,7 @@ void free_cnet(DevMem &mem, CNet &cn) {
     release(mem, cn.gtabs);
     release(mem, cn.sdescs);
     release(mem, cn.sblocks);
+    release(mem, cn.slevels);
     release(mem, cn.arena);
     release(mem, cn.tables);
     release(mem, cn.vidx_dev);
@@ -1266,6 +1269,7 @@ int schedule_small(DevMem &mem, CNet &cn) {
     std::vector<tnk::GemmParams> descs;
     std::vector<int2> blocks;
     cp.small_off.assign(1, 0);
+    cp.small_run.clear();
     for (int skip = 0; skip < 2; skip++) {
         std::vector<char> done(cn.tree.nodes.size(), 0);
         std::vector<int> todo;
@@ -1275,13 +1279,20 @@ int schedule_small(DevMem &mem, CNet &cn) {
         for (int i : todo) done[cn.steps[i].c] = 0;
         std::vector<int> &out = cp.sched[skip];
         out.clear();
+        bool chain = false;  // the last item is a run of levels that fit a chain
         while (!todo.empty()) {
             std::vector<int> ready, rest;
             for (int i : todo) {
                 const Step &s = cn.steps[i];
                 (cp.small[i] && done[s.a] && done[s.b] ? ready : rest).push_back(i);
             }
-            if (ready.size() > 1 || (ready.size() == 1 && cp.gd_off[ready[0] + 1] > cp.gd_off[ready[0]])) {
+            // one ready step alone: a small launch too if it is tiny (it may join a chain) or would
+            // need a gather launch
+            auto alone = [&](int i) {
+                const Step &s = cn.steps[i];
+                return cp.gd_off[i + 1] > cp.gd_off[i] || (cp.nver[s.c] << (s.nbat + s.nm + s.nn)) <= kSmallAlone;
+            };
+            if (ready.size() > 1 || (ready.size() == 1 && alone(ready[0]))) {
                 for (int i : ready) {
                     const Step &s = cn.steps[i];
                     tnk::GemmParams p;
@@ -1294,8 +1305,17 @@ int schedule_small(DevMem &mem, CNet &cn) {
                         blocks.push_back(make_int2((int)descs.size(), (int)o));
                     descs.push_back(p);
                 }
-                out.push_back(-(int)cp.small_off.size());
-                cp.small_off.push_back(blocks.size());
+                // a level that fits a chain joins the chain of the level just before it
+                const int l = (int)cp.small_off.size() - 1, nb = (int)blocks.size() - cp.small_off[l];
+                cp.small_off.push_back((int)blocks.size());
+                const bool fits = nb <= tnk::kChainBlocks;
+                if (fits && chain && !out.empty() && out.back() < 0) {
+                    cp.small_run.back()[1]++;
+                } else {
+                    cp.small_run.push_back({l, 1});
+                    out.push_back(-(int)cp.small_run.size());
+                }
+                chain = fits;
             } else if (ready.size() == 1) {
                 out.push_back(ready[0]);
             } else {
@@ -1310,6 +1330,9 @@ int schedule_small(DevMem &mem, CNet &cn) {
     if (descs.empty()) return TN_OK;
     RC(ensure(mem, cn.sdescs, descs.size() * sizeof(tnk::GemmParams)));
     RC(ensure(mem, cn.sblocks, blocks.size() * sizeof(int2)));
+    RC(ensure(mem, cn.slevels, cp.small_off.size() * sizeof(int)));
+    CK(cudaMemcpyAsync(cn.slevels.p, cp.small_off.data(), cp.small_off.size() * sizeof(int), cudaMemcpyHostToDevice,
+                       mem.stream));
     CK(cudaMemcpyAsync(cn.sdescs.p, descs.data(), descs.size() * sizeof(tnk::GemmParams), cudaMemcpyHostToDevice,
                        mem.stream));
     CK(cudaMemcpyAsync(cn.sblocks.p, blocks.data(), blocks.size() * sizeof(int2), cudaMemcpyHostToDevice, mem.stream));
@@ -1394,11 +1417,16 @@ int execute(CNet &cn, const uint64_t *d_closed, bool skip_beta_free, double2 *ou
     const size_t n_items = grouped ? sched.size() : cn.steps.size();
     for (size_t it = 0; it < n_items; it++) {
         if (grouped && sched[it] < 0) {
-            const size_t g = (size_t)(-1 - sched[it]);
+            const auto run = cn.cp.small_run[(size_t)(-1 - sched[it])];
             if (!d_closed && cn.net.n_closed > 0) { tn_set_error("execute: batch patterns missing"); return TN_EINVAL; }
-            tnk::small_steps<<<(unsigned)(cn.cp.small_off[g + 1] - cn.cp.small_off[g]), tnk::kSmallBlock, 0, st>>>(
-                static_cast<const tnk::GemmParams *>(cn.sdescs.p),
-                static_cast<const int2 *>(cn.sblocks.p) + cn.cp.small_off[g], d_closed);
+            const auto *descs = static_cast<const tnk::GemmParams *>(cn.sdescs.p);
+            const int2 *blocks = static_cast<const int2 *>(cn.sblocks.p);
+            const int b0 = cn.cp.small_off[run[0]], b1 = cn.cp.small_off[run[0] + run[1]];
+            if (run[1] > 1)
+                tnk::small_chain<<<tnk::kChainCluster, tnk::kChainGroups * tnk::kSmallBlock, 0, st>>>(
+                    descs, blocks, static_cast<const int *>(cn.slevels.p) + run[0], run[1], d_closed);
+            else
+                tnk::small_steps<<<(unsigned)(b1 - b0), tnk::kSmallBlock, 0, st>>>(descs, blocks + b0, d_closed);
             CK(cudaGetLastError());
             continue;
         }

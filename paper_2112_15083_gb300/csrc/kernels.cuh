@@ -331,48 +331,110 @@ __global__ void __launch_bounds__(32 * kRowWarps) cgemm_rowstage(GemmParams p) {
 // contiguous in the stored form, else per element.  Whole calls: that circuit 127 -> 86 us,
 // 20 qubits in split bf16 (92 steps) 501 -> 264 us.
 constexpr int kSmallBlock = 128;
-__global__ void __launch_bounds__(kSmallBlock) small_steps(const GemmParams *descs, const int2 *blocks,
-                                                           const uint64_t *closed_bits) {
-    __shared__ GemmParams p;
-    const int2 bl = blocks[blockIdx.x];
-    static_assert(sizeof(GemmParams) % 4 == 0, "copied as words");
-    for (int i = threadIdx.x; i < (int)(sizeof(GemmParams) / 4); i += kSmallBlock)
-        reinterpret_cast<uint32_t *>(&p)[i] = reinterpret_cast<const uint32_t *>(descs + bl.x)[i];
-    __syncthreads();
-    const long long o = (long long)bl.y + threadIdx.x;
-    if (o >= p.nver << (p.lbat + p.lm + p.ln)) return;
+// One output of a small step: what can be worked out before the operands exist.
+struct SmallWork {
+    const float2 *A, *B;  // the operands' rows (null: no output, or elements decoded one by one)
+    long long o, off;     // output, its position in C
+    long long v;
+    bool any;
+};
+__device__ __forceinline__ SmallWork small_prepare(const GemmParams &p, long long o, const uint64_t *closed_bits) {
+    SmallWork w = {nullptr, nullptr, o, 0, 0, o < p.nver << (p.lbat + p.lm + p.ln)};
+    if (!w.any) return w;
     const long long n = o & ((1LL << p.ln) - 1), m = (o >> p.ln) & ((1LL << p.lm) - 1);
-    const long long bat = (o >> (p.ln + p.lm)) & ((1LL << p.lbat) - 1), v = o >> (p.lbat + p.lm + p.ln);
-    const int K = 1 << p.lk;
+    const long long bat = (o >> (p.ln + p.lm)) & ((1LL << p.lbat) - 1);
+    w.v = o >> (p.lbat + p.lm + p.ln);
     const long long ea = ((bat << p.lm) | m) << p.lk, eb = ((bat << p.ln) | n) << p.lk;
     auto rows = [&](const GatherDesc *g) { return !g || (g->lb ? g->pos_beta[g->lb - 1] : g->nbits) >= p.lk; };
-    float2 acc = make_float2(0.f, 0.f);
     if (rows(p.gA) && rows(p.gB)) {
-        const float2 *A = p.gA ? reinterpret_cast<const float2 *>(p.gA->src) + gather_src(*p.gA, ea, closed_bits)
-                               : static_cast<const float2 *>(p.ptrA[v]) + ea;
-        const float2 *B = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, eb, closed_bits)
-                               : static_cast<const float2 *>(p.ptrB[v]) + eb;
+        w.A = p.gA ? reinterpret_cast<const float2 *>(p.gA->src) + gather_src(*p.gA, ea, closed_bits)
+                   : static_cast<const float2 *>(p.ptrA[w.v]) + ea;
+        w.B = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, eb, closed_bits)
+                   : static_cast<const float2 *>(p.ptrB[w.v]) + eb;
+    }
+    w.off = scatter_bits(bat, p.pos_bat, p.lbat) + scatter_bits(m, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln);
+    return w;
+}
+// Operands are read past L1: in a chain another SM wrote them.
+__device__ __forceinline__ void small_finish(const GemmParams &p, const SmallWork &w, const uint64_t *closed_bits) {
+    if (!w.any) return;
+    const int K = 1 << p.lk;
+    float2 acc = make_float2(0.f, 0.f);
+    if (w.A) {
         if (K >= 2) {
-#pragma unroll 4
+#pragma unroll 8
             for (int k = 0; k < K; k += 2) {
-                const float4 a = *reinterpret_cast<const float4 *>(A + k), b = *reinterpret_cast<const float4 *>(B + k);
+                const float4 a = __ldcg(reinterpret_cast<const float4 *>(w.A + k)), b = __ldcg(reinterpret_cast<const float4 *>(w.B + k));
                 acc = cfma(make_float2(a.x, a.y), make_float2(b.x, b.y), acc);
                 acc = cfma(make_float2(a.z, a.w), make_float2(b.z, b.w), acc);
             }
         } else {
-            acc = cfma(A[0], B[0], acc);
+            acc = cfma(__ldcg(w.A), __ldcg(w.B), acc);
         }
     } else {
+        const long long n = w.o & ((1LL << p.ln) - 1), bm = w.o >> p.ln;
+        const long long ea = (bm & ((1LL << (p.lbat + p.lm)) - 1)) << p.lk;
+        const long long eb = ((((bm >> p.lm) & ((1LL << p.lbat) - 1)) << p.ln) | n) << p.lk;
         for (int k = 0; k < K; k++) {
-            const float2 a = p.gA ? reinterpret_cast<const float2 *>(p.gA->src)[gather_src(*p.gA, ea + k, closed_bits)]
-                                  : static_cast<const float2 *>(p.ptrA[v])[ea + k];
-            const float2 b = p.gB ? reinterpret_cast<const float2 *>(p.gB->src)[gather_src(*p.gB, eb + k, closed_bits)]
-                                  : static_cast<const float2 *>(p.ptrB[v])[eb + k];
-            acc = cfma(a, b, acc);
+            const float2 *a = p.gA ? reinterpret_cast<const float2 *>(p.gA->src) + gather_src(*p.gA, ea + k, closed_bits)
+                                   : static_cast<const float2 *>(p.ptrA[w.v]) + ea + k;
+            const float2 *b = p.gB ? reinterpret_cast<const float2 *>(p.gB->src) + gather_src(*p.gB, eb + k, closed_bits)
+                                   : static_cast<const float2 *>(p.ptrB[w.v]) + eb + k;
+            acc = cfma(__ldcg(a), __ldcg(b), acc);
         }
     }
-    store_c(p, v, scatter_bits(bat, p.pos_bat, p.lbat) + scatter_bits(m, p.pos_m, p.lm) + scatter_bits(n, p.pos_n, p.ln),
-            acc);
+    store_c(p, w.v, w.off, acc);
+}
+// A step's parameters into shared memory, by the kSmallBlock threads tid = 0 ..
+__device__ __forceinline__ void small_load(GemmParams *p, const GemmParams *d, int tid) {
+    static_assert(sizeof(GemmParams) % 4 == 0, "copied as words");
+    for (int i = tid; i < (int)(sizeof(GemmParams) / 4); i += kSmallBlock)
+        reinterpret_cast<uint32_t *>(p)[i] = reinterpret_cast<const uint32_t *>(d)[i];
+}
+__global__ void __launch_bounds__(kSmallBlock) small_steps(const GemmParams *descs, const int2 *blocks,
+                                                           const uint64_t *closed_bits) {
+    __shared__ GemmParams p;
+    const int2 bl = blocks[blockIdx.x];
+    small_load(&p, descs + bl.x, threadIdx.x);
+    __syncthreads();
+    small_finish(p, small_prepare(p, (long long)bl.y + threadIdx.x, closed_bits), closed_bits);
+}
+
+// Consecutive small launches as one: a cluster of eight blocks runs them in turn, with a
+// cluster barrier between them in place of the end of one launch and the start of the next.
+// Launch i is blocks [level[i], level[i + 1]), at most kChainBlocks of them, one per group of
+// kSmallBlock threads.  What a launch reads that no launch writes (its steps' parameters,
+// pointers, patterns) is read between the two halves of the barrier before it, so a launch
+// costs the barrier, one read of the operands and the products.  12 qubits, 33 steps, a whole
+// call: 86 -> 60 us.
+constexpr int kChainCluster = 8, kChainGroups = 8, kChainBlocks = kChainCluster * kChainGroups;
+__global__ void __cluster_dims__(kChainCluster, 1, 1) __launch_bounds__(kChainGroups *kSmallBlock)
+    small_chain(const GemmParams *descs, const int2 *blocks, const int *level, int n_levels, const uint64_t *closed_bits) {
+    __shared__ GemmParams p[2][kChainGroups];
+    const int grp = threadIdx.x / kSmallBlock, tid = threadIdx.x % kSmallBlock;
+    const int task = blockIdx.x + grp * kChainCluster;
+    auto prepare = [&](int i) {
+        SmallWork w = {nullptr, nullptr, 0, 0, 0, false};
+        if (i < n_levels) {
+            const int b = level[i] + task;
+            if (b < level[i + 1]) {
+                const int2 bl = blocks[b];
+                small_load(&p[i & 1][grp], descs + bl.x, tid);
+                asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(kSmallBlock) : "memory");
+                w = small_prepare(p[i & 1][grp], (long long)bl.y + tid, closed_bits);
+            }
+        }
+        return w;
+    };
+    SmallWork w = prepare(0);
+    for (int i = 0; i < n_levels; i++) {
+        small_finish(p[i & 1][grp], w, closed_bits);
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        w = prepare(i + 1);
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
 }
 
 // mbarrier primitives (shared-memory barriers with transaction counts).
