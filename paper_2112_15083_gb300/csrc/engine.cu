@@ -747,16 +747,20 @@ int default_variant(const CNet &cn, size_t si) {
         return s.nn <= 5 ? kVarTc32 : kVarTc128;
     }
     if (std::min(s.nm, s.nn) == 6 && std::max(s.nm, s.nn) == 6 && small_fits(s, (size_t)cn.elem)) return kVarSmall;
-    if (std::min(s.nm, s.nn) <= 5 && s.nk <= 6) return kVarRow;
-    // the largest tile that both sides fill
+    // as for the stacked tensor-core tiles, where the step amortises building the stack list
+    if (rowstack_fits(cn, si) && s.flops_per_version >= 1e9) return kVarRowStack;
     const int lo = std::min(s.nm, s.nn), hi = std::max(s.nm, s.nn);
-    if (lo >= 6 && hi >= 7) return 128064;
-    if (lo >= 5 && hi >= 7) return 128032;
-    if (lo >= 6) return 64064;
-    if (lo >= 5 && hi >= 6) return 64032;
-    if (lo >= 5) return 32032;
-    if (lo == 4 && hi >= 7) return hi >= 8 ? 256016 : 128016;
-    if (hi >= 8) return lo == 3 ? 256008 : 256004;
+    const long long per = cn.cp.nver[s.c] << s.nbat;  // products
+    // the row kernel takes 256 rows per block: with fewer blocks than SMs its threads' long
+    // serial rows set the time ((0, 13, 5, 5): 32 blocks, 36 us), so such steps go to tiles
+    if (lo <= 5 && s.nk <= 6 && (lo <= 1 || (per << hi) >= 256LL * num_sms())) return kVarRow;
+    // the largest tile that both sides fill and that makes two blocks for every SM (a 128 x 64
+    // tile is 33 us of one SM even for a small K; (4, 9, 5, 7) x 3 versions on 192 blocks of
+    // 128 x 32: 37 us), else the smallest tile
+    for (auto &t : kTiles) {
+        const int ltm = __builtin_ctz(t[0]), ltn = __builtin_ctz(t[1]);
+        if (hi >= ltm && lo >= ltn && (per << (hi - ltm + lo - ltn)) >= 2LL * num_sms()) return t[0] * 1000 + t[1];
+    }
     return 16016;
 }
 
