@@ -159,6 +159,7 @@ struct CNet {
     long long tc_stall = 0;    // tests only: tensor-core launches first wait this many cycles
                                // on a barrier nothing arrives on (see tn_plan_test_stall)
     DBuf err;                  // device error word of the bounded waits
+    bool waits = false;        // some call plan so far launches kernels with bounded waits
     int *d_err = nullptr;
     // CUDA graphs of one execution (index: stem reuse off / on), valid for the current
     // call plan and the (closed-pattern, output) buffers they were captured with
@@ -654,6 +655,8 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
     cp.valid = true;
     cn.cp = std::move(cp);
     cn.variant.assign(cn.steps.size(), -1);
+    for (size_t i = 0; i < cn.steps.size(); i++)
+        cn.waits |= (!cn.use_tc.empty() && cn.use_tc[i]) || skinny_fits(cn, cn.steps[i]);
     const int rc = schedule_small(mem, cn);
     if (rc != TN_OK) cn.cp.valid = false;
     return rc;
@@ -1676,9 +1679,13 @@ int ensure_variant(DevMem &mem, CNet &cn, uint64_t E) {
 }
 
 
-// After a synchronising call: a bounded device wait that gave up is reported once.
+// The end of a synchronising call: waits for the stream; a bounded device wait that gave up is
+// reported once (plans without such kernels have no word to read back).
 int check_err(CNet &cn, cudaStream_t st) {
-    if (!cn.d_err) return TN_OK;
+    if (!cn.d_err || !cn.waits) {
+        CK(cudaStreamSynchronize(st));
+        return TN_OK;
+    }
     int h = 0;
     CK(cudaMemcpyAsync(&h, cn.d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -2078,7 +2085,7 @@ int tn_contract(tn_plan_h p, const uint64_t *slices, int64_t n_slices, const uin
     const bool dev = flags & TN_DEVICE_BUFFERS;
     for (long long g0 = 0; g0 < n_batches; g0 += T) {
         long long nb = std::min<long long>(T, n_batches - g0);
-        CK(cudaMemsetAsync(p->d_closed.p, 0, T * sizeof(uint64_t), st));
+        if (nb < T || p->closed.empty()) CK(cudaMemsetAsync(p->d_closed.p, 0, T * sizeof(uint64_t), st));
         if (!p->closed.empty())
             CK(cudaMemcpyAsync(p->d_closed.p, closed_bits + g0, nb * sizeof(uint64_t),
                                dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
@@ -2086,7 +2093,6 @@ int tn_contract(tn_plan_h p, const uint64_t *slices, int64_t n_slices, const uin
         CK(cudaMemcpyAsync(amps + 2 * g0 * NA, p->d_amps.p, nb * NA * sizeof(double2),
                            dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     }
-    CK(cudaStreamSynchronize(st));
     return check_err(p->amp, st);
 }
 
@@ -2145,7 +2151,6 @@ int tn_xeb(tn_plan_h p, const uint64_t *slices, int64_t n_slices, const uint64_t
     double sum = 0.0;
     CK(cudaMemcpyAsync(&sum, part + tnk::kNormGrid, sizeof(double), cudaMemcpyDeviceToHost, st));
     if (amps) CK(cudaMemcpyAsync(amps, xa, N * sizeof(double2), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
     RC(check_err(p->amp, st));
     *xeb = std::ldexp(sum, n) / (double)N - 1.0;
     return TN_OK;
