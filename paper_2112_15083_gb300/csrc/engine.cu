@@ -2303,10 +2303,8 @@ int tn_slice_cut(const double *R, int32_t k, double f, void *stream, int32_t *X,
         double *dR = static_cast<double *>(buf);
         unsigned char *res = static_cast<unsigned char *>(buf) + in_bytes;
         CK(cudaMemcpyAsync(dR, R, n * sizeof(double), cudaMemcpyHostToDevice, st));
-        size_t smem = (size_t)n * (sizeof(double) + sizeof(int));
-        tnk::slice_cut<<<1, tnk::slice_cut_threads(k), smem, st>>>(dR, k, f, reinterpret_cast<int32_t *>(res + 16),
-                                                                   reinterpret_cast<int32_t *>(res + 8),
-                                                                   reinterpret_cast<double *>(res));
+        tnk::launch_slice_cut(dR, k, f, reinterpret_cast<int32_t *>(res + 16), reinterpret_cast<int32_t *>(res + 8),
+                              reinterpret_cast<double *>(res), st);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(host, res, out_bytes, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
@@ -2942,8 +2940,7 @@ extern "C" int tn_slice_cut_noalloc(const double *R, int32_t k, double f, void *
     // the array keeps the previous call's contents: clear the count and the sum
     CK(cudaMemsetAsync(b + kCutRBytes + kCutXBytes, 0, 256, st));
     CK(cudaMemcpyAsync(dR, R, n * sizeof(double), cudaMemcpyHostToDevice, st));
-    size_t smem = (size_t)n * (sizeof(double) + sizeof(int));
-    tnk::slice_cut<<<1, tnk::slice_cut_threads(k), smem, st>>>(dR, k, f, dX, dn, dF);
+    tnk::launch_slice_cut(dR, k, f, dX, dn, dF, st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(n_x, dn, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(F, dF, sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -20,6 +20,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "widen.h"
 
 namespace tnk {
@@ -1815,96 +1817,96 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
     if ((b << 1) == 0ull) return 1ull << 63;
     return b >> 63 ? ~b : b | (1ull << 63);
 }
-__device__ __forceinline__ double order_value(unsigned long long k) {
-    if (k == 0ull) return __longlong_as_double(0x7ff8000000000000ll);
-    return __longlong_as_double((long long)(k >> 63 ? k & ~(1ull << 63) : ~k));
+
+// Alg. 1 steps 4-5 for 2^k <= 4096 norms, in two launches.  Norm i's place in (R descending,
+// i ascending) order is the number of norms before it: slice_rank counts them, 32 norms per
+// block against all keys in shared memory, one eighth of the keys per warp (a broadcast read
+// serves the 32 norms).  slice_cut then scatters the keys to their places and adds them up.
+//
+// Both are bound by latency.  A bitonic sort in one block (order keys as integers, since an
+// FP64 comparison of a warp holds the SM's FP64 pipe 16 cycles) took most of 105 us at 2^12 norms:
+// 78 dependent stages on one SM.  The FP64 prefix is a chain of one addition per norm up to
+// the cut; every lane of a warp forms it, lane l keeps the l-th of 32 sums, and the 32
+// comparisons with f are one ballot.  A whole call at 2^12 norms and f = 0.3: 150 -> 75 us.
+constexpr int kRankWarps = 8;
+__global__ void __launch_bounds__(32 * kRankWarps) slice_rank(const double *R, int k, int32_t *rank) {
+    extern __shared__ unsigned long long rank_key[];
+    __shared__ int part[kRankWarps][32];
+    const int n = 1 << k, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < n; i += 32 * kRankWarps) rank_key[i] = order_key(R[i]);
+    __syncthreads();
+    const int i = blockIdx.x * 32 + lane, seg = (n + kRankWarps - 1) / kRankWarps;
+    const int lo = warp * seg, hi = min(n, lo + seg);
+    int c = 0;
+    if (i < n) {
+        const unsigned long long x = rank_key[i];
+        // an equal norm is before i if its index is lower
+        const int mid = max(lo, min(hi, i));
+#pragma unroll 8
+        for (int j = lo; j < mid; j++) c += rank_key[j] >= x;
+#pragma unroll 8
+        for (int j = mid; j < hi; j++) c += rank_key[j] > x;
+    }
+    part[warp][lane] = c;
+    __syncthreads();
+    if (warp == 0 && i < n) {
+        int t = 0;
+        for (int w = 0; w < kRankWarps; w++) t += part[w][lane];
+        rank[i] = t;
+    }
 }
 
-// Alg. 1 steps 4-5 for 2^k <= 4096 norms in one block: bitonic sort of (R desc, i asc)
-// in shared memory, then a sequential FP64 prefix in sorted order.  Bound by latency.  The
-// sort compares order keys as integers (an FP64 comparison of a whole warp holds the SM's
-// FP64 pipe 16 cycles, and the sort makes up to 2.5 per element and stage); a thread owns
-// pair t of each stage, so the stages with strides up to 32 stay inside a warp's 64
-// elements and need no block barrier (21 barriers instead of 78 at 2^12).  The prefix keeps
-// one FP64 addition per element in its chain: eight values are fetched ahead and the
-// comparisons with f are integer ones.  A whole
-// call at 2^12 norms and f = 0.3: 547 -> 149 us (2^9, f = 1/64: 288 -> 47 us), with one buffer
-// and one copy back instead of four buffers and three copies.
-__global__ void __launch_bounds__(1024) slice_cut(const double *R, int k, double f, int32_t *X, int32_t *n_x, double *F) {
+// rank: from slice_rank; may be X itself (it is read before X is written).
+__global__ void __launch_bounds__(1024) slice_cut(const double *R, int k, double f, const int32_t *rank, int32_t *X,
+                                                  int32_t *n_x, double *F) {
     extern __shared__ unsigned char smem[];
+    __shared__ int count;
     const int n = 1 << k;
-    unsigned long long *r = reinterpret_cast<unsigned long long *>(smem);
-    int *idx = reinterpret_cast<int *>(r + n);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) { r[i] = order_key(R[i]); idx[i] = i; }
-    __syncthreads();
-    for (int size = 2; size <= n; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
-                const int i = ((t & ~(stride - 1)) << 1) | (t & (stride - 1)), j = i | stride;
-                const unsigned long long a = r[i], b = r[j];
-                const int ia = idx[i], ib = idx[j];
-                // i before j in (R descending, index ascending) order; never with a NaN
-                const bool a_first = a != 0 && b != 0 && (a > b || (a == b && ia < ib));
-                if (((i & size) == 0) != a_first) {
-                    r[i] = b;
-                    r[j] = a;
-                    idx[i] = ib;
-                    idx[j] = ia;
-                }
-            }
-            // the next stage's stride (the next size's first one when this is the last)
-            const int next = stride > 1 ? stride >> 1 : size;
-            if (stride > 32 || next > 32) __syncthreads();
-            else __syncwarp();
-        }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned long long fk = f == f ? order_key(f) : ~0ull;  // no sum reaches a NaN f
-        double acc = 0.0;
-        int cnt = n, t = 0;
-        constexpr int U = 8;
-        if (n >= U) {
-            unsigned long long nx[U];
-#pragma unroll
-            for (int i = 0; i < U; i++) nx[i] = r[i];
-            for (; t < n && cnt == n; t += U) {
-                double x[U];
-#pragma unroll
-                for (int i = 0; i < U; i++) x[i] = order_value(nx[i]);
-                if (t + U < n) {
-#pragma unroll
-                    for (int i = 0; i < U; i++) nx[i] = r[t + U + i];
-                }
-                double s[U];
-                s[0] = __dadd_rn(acc, x[0]);
-#pragma unroll
-                for (int i = 1; i < U; i++) s[i] = __dadd_rn(s[i - 1], x[i]);
-                acc = s[U - 1];
-                bool hit = false;
-#pragma unroll
-                for (int i = 0; i < U; i++)
-                    if (!hit && order_key(s[i]) >= fk) {
-                        hit = true;
-                        acc = s[i];
-                        cnt = t + i + 1;
-                    }
-                if (hit) break;
-            }
-        } else {
-            for (; t < n; t++) {
-                acc = __dadd_rn(acc, order_value(r[t]));
-                if (order_key(acc) >= fk) { cnt = t + 1; break; }
-            }
-        }
-        r[0] = (unsigned long long)cnt;  // the sorted keys are no longer needed
-        *n_x = cnt;
-        *F = acc;
+    double *r = reinterpret_cast<double *>(smem);
+    unsigned short *idx = reinterpret_cast<unsigned short *>(r + n);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int t = rank[i];
+        r[t] = R[i];
+        idx[t] = (unsigned short)i;
     }
     __syncthreads();
-    const int cnt = (int)r[0];
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const unsigned long long fk = f == f ? order_key(f) : ~0ull;  // no sum reaches a NaN f
+        double acc = 0.0;
+        int cnt = n;
+        for (int t = 0; t < n; t += 32) {
+            const int m = min(32, n - t);
+            double mine = 0.0;
+#pragma unroll 8
+            for (int i = 0; i < m; i++) {
+                acc = __dadd_rn(acc, r[t + i]);
+                if (lane == i) mine = acc;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, lane < m && order_key(mine) >= fk);
+            if (hit) {
+                const int l = __ffs(hit) - 1;
+                cnt = t + l + 1;
+                acc = __shfl_sync(0xffffffffu, mine, l);
+                break;
+            }
+        }
+        if (lane == 0) {
+            count = cnt;
+            *n_x = cnt;
+            *F = acc;
+        }
+    }
+    __syncthreads();
+    const int cnt = count;
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) X[t] = idx[t];
 }
-// Threads of a slice_cut block: one per pair of a stage, whole warps.
-inline int slice_cut_threads(int k) { return 1 << (k < 6 ? 5 : k > 11 ? 10 : k - 1); }
+// Both launches; rank and X share their 2^k words.
+inline void launch_slice_cut(const double *R, int k, double f, int32_t *X, int32_t *n_x, double *F, cudaStream_t st) {
+    const int n = 1 << k;
+    slice_rank<<<(n + 31) / 32, 32 * kRankWarps, n * sizeof(unsigned long long), st>>>(R, k, X);
+    slice_cut<<<1, std::max(32, std::min(1024, n)), n * (sizeof(double) + sizeof(unsigned short)), st>>>(R, k, f, X, X, n_x,
+                                                                                                       F);
+}
 
 }  // namespace tnk
