@@ -1475,133 +1475,183 @@ __global__ void __launch_bounds__(256) norm_total(const double *partial, double 
 
 // ---------------------------------------------------------------- top-N selection (XEB spoofing)
 
-// key[i] = the bit pattern of p_i = re*re + im*im in FP64 (rounded products, no fused
-// multiply-add): non-negative doubles order like their bit patterns.
-__global__ void spoof_keys(const double2 *a, long long n, unsigned long long *key) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const double p = __dadd_rn(__dmul_rn(a[i].x, a[i].x), __dmul_rn(a[i].y, a[i].y));
-        key[i] = (unsigned long long)__double_as_longlong(p);
-    }
-}
-
-// Histogram of the 8-bit digit at `shift` over the keys whose bits above it equal `prefix`
-// (under `mask`): one shared histogram per block, added to hist[256].
-__global__ void __launch_bounds__(256) digit_hist(const unsigned long long *key, long long n, unsigned long long mask,
-                                                  unsigned long long prefix, int shift, unsigned int *hist) {
-    __shared__ unsigned int h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const unsigned long long k = key[i];
-        if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
-}
-
-constexpr int kSelBlock = 1024;  // keys per selection block (one per thread)
-
-// Exclusive rank of this thread's flag among the block's flags, and the block's total.
-__device__ __forceinline__ unsigned int block_rank(bool f, unsigned int *warp_tot, unsigned int &total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned int b = __ballot_sync(0xffffffffu, f);
-    const unsigned int in_warp = __popc(b & ((1u << lane) - 1u));
-    if (lane == 0) warp_tot[warp] = __popc(b);
-    __syncthreads();
-    unsigned int before = 0;
-    total = 0;
-    for (int w = 0; w < kSelBlock / 32; w++) {
-        if (w < warp) before += warp_tot[w];
-        total += warp_tot[w];
-    }
-    __syncthreads();  // warp_tot is reused by the next call
-    return before + in_warp;
-}
-
-// Per block of kSelBlock consecutive keys: how many exceed the threshold and how many equal it.
-__global__ void __launch_bounds__(kSelBlock) sel_counts(const unsigned long long *key, long long n,
-                                                        unsigned long long thr, unsigned int *gt, unsigned int *eq) {
-    __shared__ unsigned int wt[kSelBlock / 32];
-    const long long i = (long long)blockIdx.x * kSelBlock + threadIdx.x;
-    const unsigned long long k = i < n ? key[i] : 0ull;
-    unsigned int tg, te;
-    block_rank(i < n && k > thr, wt, tg);
-    block_rank(i < n && k == thr, wt, te);
-    if (threadIdx.x == 0) {
-        gt[blockIdx.x] = tg;
-        eq[blockIdx.x] = te;
-    }
-}
-
-// In-place exclusive prefix sums of the per-block counts, in one block, chunk by chunk.
-__global__ void __launch_bounds__(kSelBlock) sel_scan(unsigned int *gt, unsigned int *eq, int nb) {
-    __shared__ unsigned int wg[kSelBlock / 32], we[kSelBlock / 32];
-    unsigned int carry_g = 0, carry_e = 0;
-    for (int c = 0; c < nb; c += kSelBlock) {
-        const int j = c + (int)threadIdx.x;
-        const unsigned int g = j < nb ? gt[j] : 0u, e = j < nb ? eq[j] : 0u;
-        // block-wide exclusive sums of g and e by warp scans (shuffles) of the counts
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        unsigned int sg = g, se = e;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned int yg = __shfl_up_sync(0xffffffffu, sg, o), ye = __shfl_up_sync(0xffffffffu, se, o);
-            if (lane >= o) {
-                sg += yg;
-                se += ye;
-            }
-        }
-        if (lane == 31) {
-            wg[warp] = sg;
-            we[warp] = se;
-        }
-        __syncthreads();
-        unsigned int bg = 0, be = 0, tg = 0, te = 0;
-        for (int w = 0; w < kSelBlock / 32; w++) {
-            if (w < warp) {
-                bg += wg[w];
-                be += we[w];
-            }
-            tg += wg[w];
-            te += we[w];
-        }
-        if (j < nb) {
-            gt[j] = carry_g + bg + sg - g;
-            eq[j] = carry_e + be + se - e;
-        }
-        carry_g += tg;
-        carry_e += te;
-        __syncthreads();  // wg / we are rewritten by the next chunk
-    }
-}
-
-// The open qubits of a batch: bit r of an in-batch index is qubit q[r].
+// Selection of the `need` largest of n <= 2^16 probabilities p_i = re*re + im*im in FP64
+// (rounded products, no fused multiply-add), ties by position, written in ascending position:
+// position i as the bitstring base | (bit r of i at qubit open.q[r]), with its p_i.
+//
+// One cluster of eight blocks holds all keys in registers (the bit patterns of non-negative
+// doubles order like the doubles).  A radix select, most significant 8-bit digit first, adds
+// the blocks' shared histograms through the cluster's shared memory and picks the digit in
+// every block alike, so the eight digits cost eight cluster barriers; then the blocks rank
+// the selected keys and write them.  Before, every digit was a launch, a copy to the host
+// and a wait, and the ranking three more launches: a whole call of 2^16 strings, N = 6553, 457
+// -> 339 us with a first form of this kernel (57 us); 34 us as it stands.
 struct OpenQubits {
     int8_t q[64];
     int n;
 };
+constexpr int kSelBlock = 1024, kSelCluster = 8, kSelKeys = 8;  // threads, blocks, keys per thread
 
-// Write the selected positions in ascending order: key > thr, or key == thr among the
-// first `need` equal ones (by position).  Position i goes out as the bitstring
-// base | (bit r of i at qubit open.q[r]) with its p_i.
-__global__ void __launch_bounds__(kSelBlock) sel_write(const unsigned long long *key, long long n,
-                                                       unsigned long long thr, long long need,
-                                                       const unsigned int *gt_off, const unsigned int *eq_off,
-                                                       unsigned long long base, OpenQubits open,
-                                                       unsigned long long *bits, double *prob) {
-    __shared__ unsigned int wt[kSelBlock / 32];
-    const long long i = (long long)blockIdx.x * kSelBlock + threadIdx.x;
-    const unsigned long long k = i < n ? key[i] : 0ull;
-    const bool g = i < n && k > thr, e = i < n && k == thr;
-    unsigned int t;
-    const unsigned int lg = block_rank(g, wt, t);
-    const unsigned int le = block_rank(e, wt, t);
-    const long long eq_before = (long long)eq_off[blockIdx.x] + le;
-    if (g || (e && eq_before < need)) {
-        const long long pos = (long long)gt_off[blockIdx.x] + lg + (eq_before < need ? eq_before : need);
-        unsigned long long b = base;
-        for (int r = 0; r < open.n; r++) b |= (unsigned long long)((i >> r) & 1) << open.q[r];
-        bits[pos] = b;
-        if (prob) prob[pos] = __longlong_as_double((long long)k);
+// Exclusive ranks of this thread's two flags among the block's flags, and the block's totals
+// (the second's in the upper halves).  Every warp scans the 32 warp totals by shuffles.
+__device__ __forceinline__ unsigned int block_rank2(bool f, bool g, unsigned int *warp_tot, unsigned int &total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned int bf = __ballot_sync(0xffffffffu, f), bg = __ballot_sync(0xffffffffu, g), below = (1u << lane) - 1u;
+    if (lane == 0) warp_tot[warp] = (unsigned int)__popc(bf) | (unsigned int)__popc(bg) << 16;
+    __syncthreads();
+    unsigned int inc = warp_tot[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    total = __shfl_sync(0xffffffffu, inc, 31);
+    const unsigned int before = __shfl_sync(0xffffffffu, inc, max(warp - 1, 0));
+    __syncthreads();  // warp_tot is reused by the next call
+    return (warp ? before : 0u) + ((unsigned int)__popc(bf & below) | (unsigned int)__popc(bg & below) << 16);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The word at this block's shared address `x`, in block `rank` of the cluster.
+__device__ __forceinline__ unsigned int cluster_load(const unsigned int *x, int rank) {
+    uint32_t remote, v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(x)), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
+    return v;
+}
+
+__global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelBlock)
+    spoof_select(const double2 *a, long long n, long long need, unsigned long long base, OpenQubits open,
+                 unsigned long long *bits, double *prob) {
+    __shared__ unsigned int hist[2][256], total[256], above[256], counts[2], wt[kSelBlock / 32];
+    __shared__ unsigned int pick, pick_above, pick_total;
+    const int tid = threadIdx.x, rank = blockIdx.x;
+    // block r holds positions [r per, (r + 1) per), kSelBlock at a time
+    const long long per = max((long long)kSelBlock, n / kSelCluster), first = rank * per;
+    unsigned long long key[kSelKeys];
+#pragma unroll
+    for (int j = 0; j < kSelKeys; j++) {
+        const long long o = (long long)j * kSelBlock + tid, i = first + o;
+        key[j] = 0ull;
+        if (o < per && i < n)
+            key[j] = (unsigned long long)__double_as_longlong(
+                __dadd_rn(__dmul_rn(a[i].x, a[i].x), __dmul_rn(a[i].y, a[i].y)));
+    }
+    auto held = [&](int j) {
+        const long long o = (long long)j * kSelBlock + tid;
+        return o < per && first + o < n;
+    };
+    unsigned long long prefix = 0, mask = 0;
+    unsigned int left = (unsigned int)need;
+    if (tid < 256) hist[0][tid] = 0;
+    __syncthreads();
+    for (int d = 0; d < 8; d++) {
+        const int shift = 56 - 8 * d, cur = d & 1;
+#pragma unroll
+        for (int j = 0; j < kSelKeys; j++)
+        {
+            // the leading digits of all keys are nearly the same: where a warp's digits are one, it
+            // adds their number at once (a match of arbitrary digits costs more than it saves)
+            const bool in = held(j) && (key[j] & mask) == prefix;
+            const unsigned int act = __ballot_sync(0xffffffffu, in);
+            if (act) {
+                const int lead = __ffs(act) - 1;
+                const unsigned int digit = (unsigned int)(key[j] >> shift) & 255u;
+                const unsigned int first_digit = __shfl_sync(0xffffffffu, digit, lead);
+                if (__all_sync(0xffffffffu, !in || digit == first_digit)) {
+                    if ((tid & 31) == lead) atomicAdd(&hist[cur][digit], (unsigned int)__popc(act));
+                } else if (in) {
+                    atomicAdd(&hist[cur][digit], 1u);
+                }
+            }
+        }
+        cluster_barrier();
+        // every block reads all histograms; the other buffer was last read before this barrier
+        if (tid < 256) {
+            unsigned int part[kSelCluster], t = 0;  // the loads are in flight together
+#pragma unroll
+            for (int r = 0; r < kSelCluster; r++) part[r] = cluster_load(&hist[cur][tid], r);
+#pragma unroll
+            for (int r = 0; r < kSelCluster; r++) t += part[r];
+            total[tid] = t;
+            hist[cur ^ 1][tid] = 0;
+        }
+        __syncthreads();
+        // above[x]: keys with a larger digit, by one warp, 8 digits per lane
+        if (tid < 32) {
+            unsigned int own = 0;
+            for (int i = 0; i < 8; i++) own += total[255 - (8 * tid + i)];
+            unsigned int inc = own;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (tid >= o) inc += y;
+            }
+            unsigned int run = inc - own;
+            for (int i = 0; i < 8; i++) {
+                above[255 - (8 * tid + i)] = run;
+                run += total[255 - (8 * tid + i)];
+            }
+        }
+        __syncthreads();
+        // the largest digit whose keys and those above reach `left` (0 if none does)
+        if (tid < 256 && above[tid] < left && (tid == 0 || above[tid] + total[tid] >= left)) {
+            pick = tid;
+            pick_above = above[tid];
+            pick_total = total[tid];
+        }
+        __syncthreads();
+        left -= pick_above;
+        prefix |= (unsigned long long)pick << shift;
+        mask |= 255ull << shift;
+        const bool whole = pick_total == left;  // every key with this prefix: lower digits don't matter
+        __syncthreads();
+        if (whole) break;
+    }
+    // selected: keys above prefix (as far as its digits go), and the first `left` equal to it
+    unsigned int g = 0, e = 0;
+#pragma unroll
+    for (int j = 0; j < kSelKeys; j++) {
+        g += __syncthreads_count(held(j) && (key[j] & mask) > prefix);
+        e += __syncthreads_count(held(j) && (key[j] & mask) == prefix);
+    }
+    if (tid == 0) {
+        counts[0] = g;
+        counts[1] = e;
+    }
+    cluster_barrier();
+    unsigned int g0 = 0, e0 = 0;  // in the blocks before this one
+    {
+        unsigned int cg[kSelCluster], ce[kSelCluster];
+#pragma unroll
+        for (int r = 0; r < kSelCluster; r++) {
+            cg[r] = cluster_load(&counts[0], r);
+            ce[r] = cluster_load(&counts[1], r);
+        }
+#pragma unroll
+        for (int r = 0; r < kSelCluster; r++)
+            if (r < rank) {
+                g0 += cg[r];
+                e0 += ce[r];
+            }
+    }
+    cluster_barrier();  // no block leaves while its counts are being read
+#pragma unroll
+    for (int j = 0; j < kSelKeys; j++) {
+        const bool gt = held(j) && (key[j] & mask) > prefix, eq = held(j) && (key[j] & mask) == prefix;
+        unsigned int t;
+        const unsigned int local = block_rank2(gt, eq, wt, t), lg = local & 0xffffu, le = local >> 16;
+        if (gt || (eq && e0 + le < left)) {
+            const unsigned int pos = g0 + lg + min(e0 + le, left);
+            const long long i = first + (long long)j * kSelBlock + tid;
+            unsigned long long b = base;
+            for (int r = 0; r < open.n; r++) b |= (unsigned long long)((i >> r) & 1) << open.q[r];
+            bits[pos] = b;
+            if (prob) prob[pos] = __longlong_as_double((long long)key[j]);
+        }
+        g0 += t & 0xffffu;
+        e0 += t >> 16;
     }
 }
 
