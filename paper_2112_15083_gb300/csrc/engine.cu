@@ -4,7 +4,7 @@
 // executes a slice set as follows: every tree node x gets one version per distinct
 // projection of the slice set on the sliced legs below x (so intermediates shared by
 // several slices are computed once); each step is one launch over all versions; the
-// root versions are summed in FP64 in slice order (Sec. I.C).  Leaves holding closed
+// root versions are summed in FP64 (Sec. I.C).  Leaves holding closed
 // output legs are re-materialised per batch group with the group's closed patterns.
 #include <algorithm>
 #include <array>

@@ -9,7 +9,7 @@
 //  * materialize: writes leaf tensors in the layout their consumer reads, fixing the
 //    sliced legs (one copy per slice value) and binding closed output legs to the
 //    batch pattern (the batch-indexed selector <b_B|).
-//  * slice_sum: FP64 sum over the slice set in slice order (Sec. I.C step 1);
+//  * slice_sum: FP64 sum over the slice set (Sec. I.C step 1), 16 values at a time in slice order;
 //    root_slice_sum: the same sum fused with a root step that runs the row kernel.
 //  * draw / sampler: Philox4x32-10 draws and the modified frugal rejection step
 //    (Sec. II.A), one warp per batch of 64.
@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "chunk_sum.h"
 #include "widen.h"
 
 namespace tnk {
@@ -1117,68 +1118,12 @@ __global__ void absmax_kernel(const void *data, long long n, int fmt, int *absma
 
 // out[e] = sum over explicit root versions v (in order) and over the 2^nfree patterns f
 // of the sliced legs carried as layout bits (ascending) of root_v[(f << nout) | e], FP64.
+// complex64 values are added 16 at a time where a version has that many (chunk_sum.h: 2^14
+// outputs of 48 values 16 -> 10 us; for the large sums see root_sum_small), else one by one;
 // complex64 inputs are widened with integer operations (exact), which leaves the FP64
 // pipe to the additions.
 __device__ __forceinline__ double slice_widen(float x) { return tn_widen(x); }
 __device__ __forceinline__ double slice_widen(double x) { return x; }
-
-// A running FP64 sum of FP32 values with two or three FP64 additions per 16 values.
-//
-// The FP64 pipe takes 2 lanes per clock and SM, so one addition per value bounds the sum
-// (2^20 outputs of 1024 complex values: 4.1 ms, 2.1 TB/s).  Here 16 values are first added in
-// FP32 without loss, split at powers of two (emax: exponent of the largest |x|):
-// hi = (s + x) - s with s = 1.5 * 2^(emax + 4) is a multiple of 2^(emax - 19), so the 16 hi
-// parts add exactly; lo = x - hi is at most 2^(emax - 20), and the lo parts add exactly if the
-// smallest |x| is within 2^17 of the largest.  Else lo is split the same way 20 bits lower:
-// its hi parts add exactly and what is left, at most 2^(emax - 40) each, in FP32 to within
-// 2^(emax - 56), below the rounding of one FP64 addition to a sum of that size.  So 16 values
-// take at most three FP64 roundings instead of 16, and where FP64 additions one by one would
-// not round at all (most slice sums), the result is theirs.  Values FP32 cannot split
-// (infinite, NaN, or a largest one outside 2^-80 .. 2^100) are added one by one.
-// 2^14 outputs of 48 values: 16 -> 10 us; for the large sums see root_sum_small.
-struct ChunkSum {
-    double acc = 0.0;
-    __device__ __forceinline__ void one(float x) { acc = __dadd_rn(acc, slice_widen(x)); }
-    __device__ __forceinline__ void add16(const float (&x)[16]) {
-        float mx = 0.f;
-        uint32_t mn = 0xffffffffu;  // smallest 2 |bits| - 1: zeros, which add nothing, come last
-#pragma unroll
-        for (int i = 0; i < 16; i++) {
-            mx = fmaxf(mx, fabsf(x[i]));
-            mn = min(mn, 2u * __float_as_uint(x[i]) - 1u);
-        }
-        if (mn == 0xffffffffu) return;  // all zero
-        // biased by 127; en is the exponent of the smallest value, or one less
-        const int ex = __float_as_int(mx) >> 23, en = (int)(mn >> 24);
-        const float s1 = __int_as_float(((ex + 4) << 23) | 0x400000);
-        float sh = 0.f, sl = 0.f;
-#pragma unroll
-        for (int i = 0; i < 16; i++) {
-            const float hi = __fsub_rn(__fadd_rn(s1, x[i]), s1);
-            sl = __fadd_rn(sl, __fsub_rn(x[i], hi));
-            sh = __fadd_rn(sh, hi);
-        }
-        if (!(ex >= 47 && ex <= 227 && sh == sh)) {
-#pragma unroll
-            for (int i = 0; i < 16; i++) one(x[i]);
-            return;
-        }
-        if (ex - en > 17) {
-            const float s2 = __int_as_float(((ex - 16) << 23) | 0x400000);
-            float sr = 0.f;
-            sl = 0.f;
-#pragma unroll
-            for (int i = 0; i < 16; i++) {
-                const float lo = __fsub_rn(x[i], __fsub_rn(__fadd_rn(s1, x[i]), s1));
-                const float h2 = __fsub_rn(__fadd_rn(s2, lo), s2);
-                sl = __fadd_rn(sl, h2);
-                sr = __fadd_rn(sr, __fsub_rn(lo, h2));
-            }
-            one(sr);
-        }
-        acc = __dadd_rn(acc, __dadd_rn(slice_widen(sh), slice_widen(sl)));
-    }
-};
 
 template <typename T>
 __global__ void slice_sum(const void *const *ptr, long long nver, int nfree, int nout, double2 *out) {
@@ -1203,7 +1148,7 @@ __global__ void slice_sum(const void *const *ptr, long long nver, int nfree, int
                     si.add16(xi);
                 }
             }
-            out[e] = make_double2(sr.acc, si.acc);
+            out[e] = make_double2(sr.total(), si.total());
             return;
         }
     }
@@ -1291,7 +1236,7 @@ constexpr int kRootTabBytes = 3;  // free patterns of up to 24 bits
 // values never pass through memory.  The host checks that p's batch, row and column bits
 // cover the positions [0, nout + nfree) once each, so every (bat, m, n) below is in range.
 template <typename T>
-__global__ void __launch_bounds__(256) root_slice_sum(GemmParams p, int nfree, int nout, double2 *out) {
+__global__ void __launch_bounds__(256, 3) root_slice_sum(GemmParams p, int nfree, int nout, double2 *out) {
     // byte tables: t*[j][b] are the batch, row and column bits of position (b << 8j) << nout
     __shared__ long long tbat[kRootTabBytes][256], tm[kRootTabBytes][256];
     __shared__ int tn[kRootTabBytes][256];
@@ -1338,7 +1283,7 @@ __global__ void __launch_bounds__(256) root_slice_sum(GemmParams p, int nfree, i
                     sr.add16(xr);
                     si.add16(xi);
                 }
-            out[e] = make_double2(sr.acc, si.acc);
+            out[e] = make_double2(sr.total(), si.total());
             return;
         }
     }
@@ -1364,7 +1309,7 @@ __global__ void __launch_bounds__(256) root_slice_sum(GemmParams p, int nfree, i
 // Now (22, 3, 5, 0) takes 1.57 ms in place of 3.4 + 4.1 ms, (20, 2, 4, 0) 0.14 in place of 0.37
 // + 0.28 ms; bound by issue (about 30 instructions per term, 16 of them the sums).
 template <int LK>
-__global__ void __launch_bounds__(256) root_sum_small(GemmParams p, int nfree, int nout, double2 *out) {
+__global__ void __launch_bounds__(256, 3) root_sum_small(GemmParams p, int nfree, int nout, double2 *out) {
     extern __shared__ uint2 root_off[];
     constexpr int K = 1 << LK;
     const int nf = 1 << nfree;
@@ -1403,25 +1348,27 @@ __global__ void __launch_bounds__(256) root_sum_small(GemmParams p, int nfree, i
             }
             return root_scaled(p, acc);
         };
-        int f = 0;
-        for (; f + 16 <= nf; f += 16) {
-            float xr[16], xi[16];
+        if (nf >= 16) {
+            for (int f = 0; f < nf; f += 16) {
+                float xr[16], xi[16];
 #pragma unroll
-            for (int i = 0; i < 16; i++) {
-                const float2 x = term(f + i);
-                xr[i] = x.x;
-                xi[i] = x.y;
+                for (int i = 0; i < 16; i++) {
+                    const float2 x = term(f + i);
+                    xr[i] = x.x;
+                    xi[i] = x.y;
+                }
+                sr.add16(xr);
+                si.add16(xi);
             }
-            sr.add16(xr);
-            si.add16(xi);
-        }
-        for (; f < nf; f++) {
-            const float2 x = term(f);
-            sr.one(x.x);
-            si.one(x.y);
+        } else {
+            for (int f = 0; f < nf; f++) {
+                const float2 x = term(f);
+                sr.acc = __dadd_rn(sr.acc, slice_widen(x.x));
+                si.acc = __dadd_rn(si.acc, slice_widen(x.y));
+            }
         }
     }
-    out[e] = make_double2(sr.acc, si.acc);
+    out[e] = make_double2(sr.total(), si.total());
 }
 
 // ---------------------------------------------------------------- sampling job
