@@ -88,8 +88,9 @@ def parse():
     ap.add_argument("--anneal", type=int, default=None,
                     help="simulated-annealing moves on the plan's tree (tn_plan_opts.anneal_iters); default: the "
                          "workload's (2000 for the 40-qubit job, where it is annealed per slice under the size cap)")
-    ap.add_argument("--fuse-root", type=int, default=0,
-                    help="1: run a row-kernel root step fused with the FP64 slice sum (tn_plan_opts.fuse_root_sum)")
+    ap.add_argument("--fuse-root", type=int, default=2, choices=(0, 1, 2),
+                    help="row-kernel root step and FP64 slice sum (tn_plan_opts.fuse_root_sum): 0 separate launches, "
+                         "1 always fused, 2 fused where the library finds it faster")
     ap.add_argument("--serve", action="store_true", help="serving run (Poisson request stream) instead of the step bench")
     ap.add_argument("--serve-window", type=float, default=60.0, help="seconds of arrivals")
     ap.add_argument("--serve-rate", type=float, default=4.0, help="requests per second")
@@ -454,7 +455,7 @@ def workload_config(args):
                             1 << log2_batches(args)),
             "qubits": q, "cycles": w["cycles"], "sliced_legs": w["n_sliced"], "batches_per_step": 1 << log2_batches(args),
             "batch_size": 64, "fidelity_target": args.fidelity, "alpha": 2.0, "order_trials": args.trials,
-            "precision": getattr(args, "precision", "c64"), "fuse_root_sum": bool(getattr(args, "fuse_root", 0)),
+            "precision": getattr(args, "precision", "c64"), "fuse_root_sum": {0: "never", 1: "always", 2: "where faster"}[getattr(args, "fuse_root", 2)],
             "anneal_iters": int(getattr(args, "anneal", 0)),
             "job": "the timed steps are the batch groups of one sampling job over one slice set",
             "l2": "flushed between timed steps; dominant operands exceed L2"}
@@ -477,7 +478,7 @@ def run_group(args, with_e2e=True, with_cpu=True):
     prec = {"c64": P.tn.PREC_C64, "bf16x2": P.tn.PREC_BF16X2}[args.precision]
     plan = P.plan(C, openq, n_auto_sliced=w["n_sliced"], log2_batches=log2_batches(args), order_trials=args.trials,
                   order_seed=0, hbm_budget_bytes=200e9, precision=prec, autotune=args.autotune,
-                  fuse_root_sum=bool(args.fuse_root), anneal_iters=args.anneal)
+                  fuse_root_sum=(False, True, None)[args.fuse_root], anneal_iters=args.anneal)
     info = plan.info()
     slices, F = plan.select(args.fidelity)
     T = 1 << log2_batches(args)
@@ -777,7 +778,7 @@ def secondary_lines(args):
     for prec in ("bf16x2", "c64"):
         a = argparse.Namespace(**vars(args))
         a.workload, a.precision, a.fidelity, a.steps, a.warmup = "grid4x7_m14", prec, 1.0, 5, 3
-        a.log2_batches, a.fuse_root, a.anneal = None, 0, 0
+        a.log2_batches, a.fuse_root, a.anneal = None, 2, 0
         line = run_group(a, with_e2e=False, with_cpu=False)
         out["grid4x7_m14_" + prec] = {
             "value": line["value"], "ms_per_step": line["ms_per_step"], "steps": a.steps, "fidelity": line["fidelity"],

@@ -154,8 +154,8 @@ struct CNet {
     const uint64_t *cur_closed = nullptr;  // batch patterns of the execution being issued
     int autotune = 1;          // 1: time the applicable variants of unseen step shapes;
                                // 0: fixed shape rules; k >= 2: variant (step + k - 2) mod count
-    int fuse_root = 0;         // run a row-kernel root step fused with the slice sum: 1 always,
-                               // 0 where the fast form applies (root_small), -1 never
+    int fuse_root = 2;         // run a row-kernel root step fused with the slice sum: 0 never, 1
+                               // always, 2 where the fast form applies (root_small)
     long long tc_stall = 0;    // tests only: tensor-core launches first wait this many cycles
                                // on a barrier nothing arrives on (see tn_plan_test_stall)
     DBuf err;                  // device error word of the bounded waits
@@ -1353,11 +1353,11 @@ int schedule_small(DevMem &mem, CNet &cn) {
 // kernel's byte tables; it is off while FP16 scales are calibrated (every node's maximum
 // is recorded from its stored values).
 long long fused_root_step(const CNet &cn) {
-    if (cn.fuse_root < 0 || cn.calibrating || cn.steps.empty() || !cn.cp.valid) return -1;
+    if (cn.fuse_root <= 0 || cn.calibrating || cn.steps.empty() || !cn.cp.valid) return -1;
     const int root = cn.tree.root;
     const size_t si = cn.steps.size() - 1;
     const Step &s = cn.steps[si];
-    if (s.c != root || (cn.fuse_root == 0 && !root_small(cn, si))) return -1;
+    if (s.c != root || (cn.fuse_root == 2 && !root_small(cn, si))) return -1;
     const int var = si < cn.variant.size() && cn.variant[si] >= 0 ? cn.variant[si] : default_variant(cn, si);
     if (var != kVarRow || cn.fmt[root] != tnk::OUT_C64) return -1;
     const int nout = (int)cn.net.out_layout.size();
@@ -1511,7 +1511,7 @@ bool resolve_variants(CNet &cn) {
             continue;
         }
         // a root that runs fused with the slice sum (row kernel) is not timed by itself
-        if (cn.fuse_root >= 0 && cn.steps[si].c == cn.tree.root && root_small(cn, si) &&
+        if (cn.fuse_root > 0 && cn.steps[si].c == cn.tree.root && root_small(cn, si) &&
             std::find(c.begin(), c.end(), kVarRow) != c.end()) {
             cn.variant[si] = kVarRow;
             continue;
@@ -1874,7 +1874,7 @@ void tn_plan_opts_default(tn_plan_opts *o) {
     o->hbm_budget_bytes = 64.0 * (1ull << 30);
     o->max_norm_flops = 2e15;
     o->autotune = 1;
-    o->fuse_root_sum = 0;
+    o->fuse_root_sum = 2;
     o->job_groups = 1;
 }
 

@@ -260,7 +260,7 @@ class Plan:
     def __init__(self, circuit: Circuit, open_qubits, sliced=None, order=None, precision=PREC_C64,
                  log2_batches=8, order_seed=0, order_trials=64, n_auto_sliced=0,
                  hbm_budget_bytes=0.0, stream=None, use_torch_allocator=True, max_norm_flops=0.0,
-                 autotune=None, max_log2_tensor=0, fuse_root_sum=False, job_groups=1, anneal_iters=0,
+                 autotune=None, max_log2_tensor=0, fuse_root_sum=None, job_groups=1, anneal_iters=0,
                  parallel_search=False):
         L = lib()
         o = PlanOpts()
@@ -277,7 +277,8 @@ class Plan:
             o.max_norm_flops = max_norm_flops
         if autotune is not None:
             o.autotune = int(autotune)
-        o.fuse_root_sum = -1 if fuse_root_sum < 0 else int(bool(fuse_root_sum))
+        if fuse_root_sum is not None:  # None: where the library finds it faster
+            o.fuse_root_sum = int(fuse_root_sum > 0)
         o.job_groups = int(job_groups)
         o.anneal_iters = int(anneal_iters)
         o.parallel_search = int(bool(parallel_search))
