@@ -91,8 +91,9 @@ typedef struct {
                                 the FP64 slice sum (Sec. I.C step 1) in one launch whose
                                 output is bit-identical to the two launches, without
                                 writing the root's per-slice values to memory.  0: separate
-                                launches; 1: always; 2 (default): where the fused kernel's
-                                fast form applies (complex64, K <= 4) */
+                                launches; 1: always; 2 (default): where it is faster (a
+                                complex64 root of K <= 4 with enough outputs for its
+                                terms) */
     int32_t job_groups;      /* batch groups per sampling job that the order search
                                 optimises for: a batch-independent step runs once per
                                 job, the others once per group; <= 1 (default): one */

@@ -155,7 +155,7 @@ struct CNet {
     int autotune = 1;          // 1: time the applicable variants of unseen step shapes;
                                // 0: fixed shape rules; k >= 2: variant (step + k - 2) mod count
     int fuse_root = 2;         // run a row-kernel root step fused with the slice sum: 0 never, 1
-                               // always, 2 where the fast form applies (root_small)
+                               // always, 2 where that is faster (root_faster)
     long long tc_stall = 0;    // tests only: tensor-core launches first wait this many cycles
                                // on a barrier nothing arrives on (see tn_plan_test_stall)
     DBuf err;                  // device error word of the bounded waits
@@ -1246,14 +1246,33 @@ int launch_slice_sum(CNet &cn, double2 *out, cudaStream_t st) {
 
 // Whether the root step si has the fused kernel's fast form: complex64, K of at most 4, at
 // most 2^12 free patterns (their offsets are a 32 KiB table) and operands of 32-bit
-// offsets.  Its bits equal those of the separate launches, and it is faster for every root
-// it accepts (no value of the root is written or read back), so it is on by default.
+// offsets.  Its bits equal those of the separate launches.
 bool root_small(const CNet &cn, size_t si) {
     const Step &s = cn.steps[si];
     const int nfree = (int)cn.tree.nodes[s.c].layout.size() - (int)cn.net.out_layout.size();
     auto bits = [&](int o) { return s.gat[o] ? (int)s.g_nbits[o] : (int)cn.tree.nodes[o ? s.b : s.a].layout.size(); };
     return cn.elem == 8 && s.nk <= 2 && nfree >= 0 && nfree <= 12 && bits(0) <= 32 && bits(1) <= 32 &&
            cn.fmt[s.a] == tnk::OUT_C64 && cn.fmt[s.b] == tnk::OUT_C64;
+}
+
+// Whether the fast form beats the separate launches.  It saves a launch (4 to 5 us) and the
+// root's values, 8 bytes written and read back per term, but a thread forms the terms of an
+// output one after the other, where the row kernel is parallel over them.  The line was
+// drawn from 248 roots of 12 to 28 qubits (fused against separate, us; (outputs, terms)
+// are powers of two): with 16 or more free patterns the terms are formed 16 at a time, and
+// outputs fill the chip from 2^12 on, K = 1: (2^12, 2^9) 51 : 65, (2^10, 2^11) 208 : 178;
+// K = 2 from 2^14: (2^14, 2^8) 61 : 79, (2^10, 2^9) 87 : 54; K = 4 from 2^16: (2^16, 2^8) 90 :
+// 131, (2^14, 2^10) 260 : 201.  Below that, and where every term is an explicit version and
+// follows the last, only short sums gain: up to 64 and 32 products, (2^6, 2^6) 11 : 17, (2^10,
+// 85 versions) 68 : 51; among the latter longer ones while the outputs fill the chip and
+// their operands stay in L2: (2^16, 170 versions) 102 : 129, (2^22, 85 versions) 4106 : 2969.
+bool root_faster(const CNet &cn, size_t si) {
+    if (!root_small(cn, si)) return false;
+    const Step &s = cn.steps[si];
+    const int nout = (int)cn.net.out_layout.size(), nfree = (int)cn.tree.nodes[s.c].layout.size() - nout;
+    const long long terms = cn.cp.root_nver << nfree, products = terms << s.nk;
+    if (nfree >= 4) return nout >= 12 + 2 * s.nk || products <= 64;
+    return (nout <= 18 && products <= 32) || (nout >= 16 && nout <= 20 && terms >= 12);
 }
 
 // The launch order with the small steps grouped: every small step whose operands exist runs in
@@ -1347,23 +1366,20 @@ int schedule_small(DevMem &mem, CNet &cn) {
     return TN_OK;
 }
 
-// The root step's index when it runs fused with the slice sum (-1: not fused).  Fusion
-// needs the row kernel on a root stored as plain complex values, batch, row and column
-// bits that cover the root layout once each, and free patterns that fit the fused
-// kernel's byte tables; it is off while FP16 scales are calibrated (every node's maximum
-// is recorded from its stored values).
-long long fused_root_step(const CNet &cn) {
-    if (cn.fuse_root <= 0 || cn.calibrating || cn.steps.empty() || !cn.cp.valid) return -1;
+// Whether step si is a root step that fuses with the slice sum when it runs the row kernel:
+// a root stored as plain complex values, batch, row and column bits that cover its layout
+// once each, free patterns that fit the fused kernel's byte tables, and a plan that asks for it.
+// Off while FP16 scales are calibrated (every node's maximum is recorded from its stored
+// values).
+bool root_fuses(const CNet &cn, size_t si) {
+    if (cn.fuse_root <= 0 || cn.calibrating || !cn.cp.valid) return false;
     const int root = cn.tree.root;
-    const size_t si = cn.steps.size() - 1;
     const Step &s = cn.steps[si];
-    if (s.c != root || (cn.fuse_root == 2 && !root_small(cn, si))) return -1;
-    const int var = si < cn.variant.size() && cn.variant[si] >= 0 ? cn.variant[si] : default_variant(cn, si);
-    if (var != kVarRow || cn.fmt[root] != tnk::OUT_C64) return -1;
+    if (s.c != root || cn.fmt[root] != tnk::OUT_C64 || (cn.fuse_root == 2 && !root_faster(cn, si))) return false;
     const int nout = (int)cn.net.out_layout.size();
     const int nfree = (int)cn.tree.nodes[root].layout.size() - nout;
-    if (nfree < 0 || nfree > 8 * tnk::kRootTabBytes || cn.cp.nver[root] != cn.cp.root_nver) return -1;
-    if (s.nbat + s.nm + s.nn != nout + nfree || nout + nfree > tnk::kMaxBits) return -1;
+    if (nfree < 0 || nfree > 8 * tnk::kRootTabBytes || cn.cp.nver[root] != cn.cp.root_nver) return false;
+    if (s.nbat + s.nm + s.nn != nout + nfree || nout + nfree > tnk::kMaxBits) return false;
     uint64_t seen = 0;
     auto mark = [&](const int8_t *pos, int n) {
         for (int i = 0; i < n; i++) {
@@ -1372,8 +1388,15 @@ long long fused_root_step(const CNet &cn) {
         }
         return true;
     };
-    if (!mark(s.pos_bat, s.nbat) || !mark(s.pos_m, s.nm) || !mark(s.pos_n, s.nn)) return -1;
-    return (long long)si;
+    return mark(s.pos_bat, s.nbat) && mark(s.pos_m, s.nm) && mark(s.pos_n, s.nn);
+}
+
+// The root step's index when it runs fused with the slice sum (-1: not fused).
+long long fused_root_step(const CNet &cn) {
+    if (cn.steps.empty()) return -1;
+    const size_t si = cn.steps.size() - 1;
+    const int var = si < cn.variant.size() && cn.variant[si] >= 0 ? cn.variant[si] : default_variant(cn, si);
+    return var == kVarRow && root_fuses(cn, si) ? (long long)si : -1;
 }
 
 // The root step (row kernel) and the FP64 slice sum in one launch: bit-identical to the
@@ -1511,7 +1534,7 @@ bool resolve_variants(CNet &cn) {
             continue;
         }
         // a root that runs fused with the slice sum (row kernel) is not timed by itself
-        if (cn.fuse_root > 0 && cn.steps[si].c == cn.tree.root && root_small(cn, si) &&
+        if (root_small(cn, si) && root_fuses(cn, si) &&
             std::find(c.begin(), c.end(), kVarRow) != c.end()) {
             cn.variant[si] = kVarRow;
             continue;

@@ -45,3 +45,34 @@ def test_fuse_root_sum_is_what_was_asked_for():
         outs.append(out)
     assert kernels == [3, 3, 3, 2, 2]  # 3: one launch with the root step, 2: a launch of its own
     assert all(np.array_equal(o, outs[0]) for o in outs)
+
+
+# a root with few outputs for its terms runs unfused by default: the fused kernel forms an
+# output's terms one after the other.  rows, cols, cycles, circuit seed, open qubits, sliced
+# legs, log2 batches, order seed; the root's (log2 outputs, free patterns, K); fused
+@pytest.mark.parametrize("case,shape,fused", [
+    ((4, 5, 9, 24, 10, 9, 0, 673), (10, 9, 1), False),
+    ((4, 4, 7, 38, 6, 8, 4, 344), (10, 8, 2), False),
+    ((4, 5, 7, 73, 4, 12, 6, 931), (10, 12, 2), False),
+    ((4, 6, 7, 48, 6, 4, 4, 739), (10, 4, 2), True),
+    ((4, 4, 6, 49, 6, 9, 6, 139), (12, 9, 0), True),
+])
+def test_default_fuses_where_the_outputs_fill_the_chip(case, shape, fused):
+    import paper_2112_15083_gb300 as P
+    rows, cols, cycles, circuit_seed, n_open, sliced, lb, order_seed = case
+    C = P.circuit_load(cg.sycamore_grid(rows, cols, cycles, seed=circuit_seed).serialize())
+    openq = cg.default_open_qubits(rows, cols, n_open)
+    cb = cg.random_closed_bits(1 << lb, rows * cols - n_open, seed=1)
+    outs, kernels = [], []
+    for fuse in (None, False, True):
+        plan = P.plan(C, openq, n_auto_sliced=sliced, log2_batches=lb, order_trials=2, order_seed=order_seed,
+                      fuse_root_sum=fuse)
+        sl = np.arange(1 << sliced, dtype=np.uint64)
+        entry, out = traced_sum(plan, sl, cb)
+        root = P.tn.plan_host(
+            C, openq, n_auto_sliced=sliced, log2_batches=lb, order_trials=2, order_seed=order_seed)[1][-1]
+        assert (n_open + lb, sum(root[:3]) - n_open - lb, root[3]) == shape
+        kernels.append(entry["kernel"])
+        outs.append(out)
+    assert kernels == [3 if fused else 2, 2, 3]
+    assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])
