@@ -230,8 +230,10 @@ int tn_select(tn_plan_h p, double f, uint64_t *slices, int64_t cap, int64_t *n_s
 
 /*
  * Host-only estimate for a slice set (no device work): device_bytes = arena + leaves +
- * per-group buffers (+ 64 MiB slack); flops_first / flops_next = algorithmic FLOPs of the
- * first batch group and of each later group (which reuses the batch-free stem).
+ * per-group buffers + 64 MiB (tables, and up to 48 MiB that an execution takes for the
+ * results of small steps where the budget has room); flops_first / flops_next =
+ * algorithmic FLOPs of the first batch group and of each later group (which reuses the
+ * batch-free stem).
  */
 int tn_plan_estimate(tn_plan_h p, const uint64_t *slices, int64_t n_slices, int64_t *device_bytes,
                      double *flops_first, double *flops_next);

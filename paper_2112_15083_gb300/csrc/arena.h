@@ -48,29 +48,21 @@ struct CallLayout {
 
 // Steps cheap enough to share a launch: a launch costs 2 to 4 us in a replayed graph, about
 // what 2^18 outputs over a short K take on the whole chip.  Their results (at most 2 MiB
-// each, 64 MiB together) are never overwritten within an execution.
+// each, 48 MiB together) are never overwritten within an execution.  The memory estimates leave
+// them out (they carry 64 MiB of slack), and an execution without room for them keeps its
+// small steps in the arena like the others and runs them one by one.
 constexpr long long kSmallOutputs = 1ll << 18, kSmallMacs = 1ll << 21, kSmallAlone = 1ll << 15;
-constexpr size_t kSmallBytes = size_t(64) << 20;
+constexpr size_t kSmallBytes = size_t(48) << 20;
 inline bool small_step(const Step &s, long long nver) {
     const int out = s.nbat + s.nm + s.nn;
     return s.nk <= 6 && out <= 18 && (nver << out) <= kSmallOutputs && (nver << (out + s.nk)) <= kSmallMacs;
 }
 
-inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64_t E, int elem,
-                 const std::vector<uint64_t> &slices, CallLayout &L) {
+// Arena offsets of a call whose versions (L.nver) are known; small: the small steps' results
+// get memory of their own in the reserved prefix.
+inline void place_call(const Tree &tree, const std::vector<Step> &steps, uint64_t E, int elem, bool small, CallLayout &L) {
     const auto &nodes = tree.nodes;
     const int NN = (int)nodes.size();
-    L.vals.assign(NN, {});
-    L.index.assign(NN, {});
-    L.nver.assign(NN, 0);
-    for (int x = 0; x < NN; x++) {
-        const uint64_t D = nodes[x].dep & E;
-        for (uint64_t s : slices) {
-            uint64_t w = s & D;
-            if (L.index[x].emplace(w, (int)L.vals[x].size()).second) L.vals[x].push_back(w);
-        }
-        L.nver[x] = (long long)L.vals[x].size();
-    }
     // arena: first fit, children released after their parent's step; beta-free
     // nodes consumed by beta steps stay alive (reused by later batch groups)
     auto tensor_bytes = [&](int x) {
@@ -116,7 +108,7 @@ inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64
     size_t small_bytes = 0;
     for (size_t i = 0; i < steps.size(); i++) {
         const Step &s = steps[i];
-        if (s.c == tree.root || !small_step(s, L.nver[s.c])) continue;
+        if (!small || s.c == tree.root || !small_step(s, L.nver[s.c])) continue;
         const size_t b = (tensor_bytes(s.c) + 255) & ~size_t(255);
         if (small_bytes + b > kSmallBytes) continue;
         small_bytes += b;
@@ -157,4 +149,28 @@ inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64
         if (nodes[s.c].beta) L.flops_beta += fl;
     }
     L.arena_bytes = std::max<size_t>(reserved + peak, 256);
+}
+
+// Versions and arena of a call; small: the small steps' results are kept apart, unless that
+// costs more than kSmallBytes (a first fit can do worse with fewer tensors).
+inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64_t E, int elem,
+                 const std::vector<uint64_t> &slices, CallLayout &L, bool small = true) {
+    const auto &nodes = tree.nodes;
+    const int NN = (int)nodes.size();
+    L.vals.assign(NN, {});
+    L.index.assign(NN, {});
+    L.nver.assign(NN, 0);
+    for (int x = 0; x < NN; x++) {
+        const uint64_t D = nodes[x].dep & E;
+        for (uint64_t s : slices) {
+            uint64_t w = s & D;
+            if (L.index[x].emplace(w, (int)L.vals[x].size()).second) L.vals[x].push_back(w);
+        }
+        L.nver[x] = (long long)L.vals[x].size();
+    }
+    place_call(tree, steps, E, elem, false, L);
+    if (!small) return;
+    const size_t least = L.arena_bytes;
+    place_call(tree, steps, E, elem, true, L);
+    if (L.arena_bytes > least + kSmallBytes) place_call(tree, steps, E, elem, false, L);
 }

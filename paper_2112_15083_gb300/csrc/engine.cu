@@ -439,7 +439,8 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
     cp.slices = slices;
     const auto &nodes = cn.tree.nodes;
     CallLayout lay;
-    layout_call(cn.tree, cn.steps, cn.E, cn.elem, slices, lay);
+    // plans that prescribe each step's variant run every step by itself (see execute)
+    layout_call(cn.tree, cn.steps, cn.E, cn.elem, slices, lay, cn.autotune < 2);
     auto &vals = lay.vals;
     auto &index = lay.index;
     cp.nver = lay.nver;
@@ -477,6 +478,7 @@ int prepare_call(DevMem &mem, CNet &cn, const std::vector<uint64_t> &slices, dou
             RC(setup_leaves(mem, cn));
         }
     }
+    if ((double)lay.arena_bytes + (double)cn.leaf_bytes > budget) place_call(cn.tree, cn.steps, cn.E, cn.elem, false, lay);
     cp.off = lay.off;
     cp.small = lay.small;
     cp.arena_bytes = lay.arena_bytes;
@@ -1741,7 +1743,8 @@ int build_cnet(const Merged &mg, CNet &cn, const tn_plan_opts &o, const int32_t 
 
 namespace {
 
-// Device bytes of one execution on slice set sl (arena, leaves, per-group buffers, slack)
+// Device bytes of one execution on slice set sl (arena, leaves, per-group buffers, and 64 MiB
+// for tables and the small steps' results)
 // and its algorithmic FLOPs for the first and each later batch group; host only.
 int estimate_call(tn_plan_s *p, const std::vector<uint64_t> &sl, int64_t *bytes, double *flops_first,
                   double *flops_next) {
@@ -1750,7 +1753,7 @@ int estimate_call(tn_plan_s *p, const std::vector<uint64_t> &sl, int64_t *bytes,
     std::vector<Step> steps;
     RC(tn_compile(p->amp.net, t, E, steps, p->amp.prec != TN_PREC_C64));
     CallLayout lay;
-    layout_call(t, steps, E, 8, sl, lay);
+    layout_call(t, steps, E, 8, sl, lay, false);
     const long long T = 1LL << p->log2T;
     if (bytes) *bytes = (int64_t)(lay.arena_bytes + 2 * p->amp.leaf_bytes + T * (64 * 16 + 64)) + (64ll << 20);
     if (flops_first) *flops_first = lay.flops;
@@ -2073,7 +2076,7 @@ int tn_plan_estimate(tn_plan_h p, const uint64_t *slices, int64_t n_slices, int6
     std::vector<Step> steps;
     RC(tn_compile(p->amp.net, t, E, steps, p->amp.prec != TN_PREC_C64));
     CallLayout lay;
-    layout_call(t, steps, E, 8, sl, lay);
+    layout_call(t, steps, E, 8, sl, lay, false);
     const long long T = 1LL << p->log2T;
     if (device_bytes)
         *device_bytes = (int64_t)(lay.arena_bytes + 2 * p->amp.leaf_bytes + T * (64 * 16 + 64)) + (64ll << 20);
