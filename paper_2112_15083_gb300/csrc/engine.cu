@@ -165,7 +165,7 @@ struct CNet {
     // call plan and the (closed-pattern, output) buffers they were captured with
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     const void *graph_key[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-    int elem = 8;  // 8: complex64, 16: complex128
+    int elem = 8;  // bytes per element (complex64, or four 16-bit planes)
     std::vector<DBuf> leaf_src, leaf_dst;
     std::vector<int> leaf_codebits;
     std::vector<std::vector<int>> leaf_sl;  // sliced legs (e) in leg order
@@ -368,7 +368,7 @@ int setup_leaves(DevMem &mem, CNet &cn) {
         cn.leaf_bytes += dst_bytes + src_bytes;
         d.src = static_cast<const double2 *>(cn.leaf_src[i].p);
         d.dst = cn.leaf_dst[i].p;
-        d.fmt = cn.elem == 8 ? cn.fmt[i] : tnk::OUT_C64;
+        d.fmt = cn.fmt[i];
         d.scale = cn.scale[i];
         static_descs.push_back(d);
     }
@@ -379,8 +379,7 @@ int setup_leaves(DevMem &mem, CNet &cn) {
         CK(cudaMemcpyAsync(tmp.b.p, static_descs.data(), static_descs.size() * sizeof(tnk::MatDesc),
                            cudaMemcpyHostToDevice, mem.stream));
         dim3 grid(4, (unsigned)static_descs.size());
-        if (cn.elem == 8) tnk::materialize<float2><<<grid, 256, 0, mem.stream>>>((const tnk::MatDesc *)tmp.b.p);
-        else tnk::materialize<double2><<<grid, 256, 0, mem.stream>>>((const tnk::MatDesc *)tmp.b.p);
+        tnk::materialize<<<grid, 256, 0, mem.stream>>>((const tnk::MatDesc *)tmp.b.p);
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(mem.stream));
     }
@@ -996,28 +995,23 @@ void row_roles(const CNet &cn, const Step &s, tnk::GemmParams &p, bool in_place)
     }
 }
 
-template <typename T>
 int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
     tnk::GemmParams p;
     RC(step_params(cn, s, p));
     const size_t si = &s - cn.steps.data();
     if (cn.trace) cn.tr_kernel[si] = var;
     if (is_tc_variant(var)) {
-        if constexpr (sizeof(T) == sizeof(float2)) {
-            if (var == kVarTc128) return launch_tc<128, 3>(cn, s, si, p, st);
-            if (var == kVarTc64) return launch_tc<64, 4>(cn, s, si, p, st);
-            if (var == kVarTcS128) return launch_tc<128, 3>(cn, s, si, p, st, true);
-            if (var == kVarTcS64) return launch_tc<64, 4>(cn, s, si, p, st, true);
-            return launch_tc<32, 5>(cn, s, si, p, st);
-        }
-        tn_set_error("tensor-core variant on a complex128 network");
-        return TN_EINVAL;
+        if (var == kVarTc128) return launch_tc<128, 3>(cn, s, si, p, st);
+        if (var == kVarTc64) return launch_tc<64, 4>(cn, s, si, p, st);
+        if (var == kVarTcS128) return launch_tc<128, 3>(cn, s, si, p, st, true);
+        if (var == kVarTcS64) return launch_tc<64, 4>(cn, s, si, p, st, true);
+        return launch_tc<32, 5>(cn, s, si, p, st);
     }
     if (var == kVarSmall) {
         // stage 2^lg batches per block in shared memory
         const int per = ((1 << s.nm) + (1 << s.nn)) * ((1 << s.nk) + 1);  // padded elements per batch
         int lg = 0;
-        while (lg < s.nbat && (size_t)(per << (lg + 1)) * sizeof(T) <= 48 * 1024 && (1 << (lg + 1 + s.nm + s.nn)) <= 4096) lg++;
+        while (lg < s.nbat && (size_t)(per << (lg + 1)) * sizeof(float2) <= 48 * 1024 && (1 << (lg + 1 + s.nm + s.nn)) <= 4096) lg++;
         tnk::SmallMap sm;
         std::memset(&sm, 0, sizeof(sm));
         sm.lg = lg;
@@ -1032,172 +1026,150 @@ int launch_variant(CNet &cn, const Step &s, cudaStream_t st, int var) {
             sm.idx[i] = (int8_t)bits[i].second.second;
         }
         const long long blocks = p.nver << (s.nbat - lg);
-        const size_t smem = (size_t)(per << lg) * sizeof(T);
-        tnk::cgemm_small<T><<<(unsigned)blocks, 256, smem, st>>>(p, sm);
+        const size_t smem = (size_t)(per << lg) * sizeof(float2);
+        tnk::cgemm_small<float2><<<(unsigned)blocks, 256, smem, st>>>(p, sm);
     } else if (var == kVarRowStage) {
         if (!rowstage_fits(cn, s)) { tn_set_error("staged row kernel: unsupported step shape"); return TN_EINVAL; }
-        if constexpr (sizeof(T) == sizeof(float2)) {
-            row_roles(cn, s, p, row_fuses(cn, si));
-            const long long rows = p.nver << (p.lbat + p.lm);
-            const int per_block = 32 * tnk::kRowWarps;
-            const size_t smem = (size_t)per_block * (8 * (1 << p.lk) + tnk::kRowPad);
-            const unsigned blocks = (unsigned)std::min<long long>((rows + per_block - 1) / per_block, 3LL * num_sms());
-            auto go = [&](auto kern) -> int {
-                CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                kern<<<blocks, per_block, smem, st>>>(p);
-                return TN_OK;
-            };
-            switch (p.ln) {
-                case 0: RC(go(tnk::cgemm_rowstage<1>)); break;
-                case 1: RC(go(tnk::cgemm_rowstage<2>)); break;
-                case 2: RC(go(tnk::cgemm_rowstage<4>)); break;
-                case 3: RC(go(tnk::cgemm_rowstage<8>)); break;
-                case 4: RC(go(tnk::cgemm_rowstage<16>)); break;
-                default: RC(go(tnk::cgemm_rowstage<32>)); break;
-            }
+        row_roles(cn, s, p, row_fuses(cn, si));
+        const long long rows = p.nver << (p.lbat + p.lm);
+        const int per_block = 32 * tnk::kRowWarps;
+        const size_t smem = (size_t)per_block * (8 * (1 << p.lk) + tnk::kRowPad);
+        const unsigned blocks = (unsigned)std::min<long long>((rows + per_block - 1) / per_block, 3LL * num_sms());
+        auto go = [&](auto kern) -> int {
+            CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            kern<<<blocks, per_block, smem, st>>>(p);
+            return TN_OK;
+        };
+        switch (p.ln) {
+            case 0: RC(go(tnk::cgemm_rowstage<1>)); break;
+            case 1: RC(go(tnk::cgemm_rowstage<2>)); break;
+            case 2: RC(go(tnk::cgemm_rowstage<4>)); break;
+            case 3: RC(go(tnk::cgemm_rowstage<8>)); break;
+            case 4: RC(go(tnk::cgemm_rowstage<16>)); break;
+            default: RC(go(tnk::cgemm_rowstage<32>)); break;
         }
     } else if (var == kVarRowStack) {
         if (!rowstack_fits(cn, si)) { tn_set_error("stacked row kernel: unsupported step shape"); return TN_EINVAL; }
-        if constexpr (sizeof(T) == sizeof(float2)) {
-            row_roles(cn, s, p, true);
-            tnk::TcGather g;
-            RC(fill_gather(cn, s, s.nn > s.nm ? 1 : 0, g));
-            const int S = tnk::kTcMaxStack;
-            int *stack = static_cast<int *>(cn.stacks.p);
-            tnk::tc_stack_build<<<1, 1024, (size_t)8 << cn.net.n_beta, st>>>(g, cn.net.n_beta, S, stack);
-            CK(cudaGetLastError());
-            // items of up to 2048 rows; the number of stacks is known on the device only
-            const long long most = (1LL << (s.nbat + p.lm - 8));
-            const unsigned blocks = (unsigned)std::min<long long>(most, 4LL * num_sms());
-            auto by_k = [&](auto n_tag) {
-                constexpr int N = decltype(n_tag)::value;
-                if (p.lk == 2) tnk::cgemm_rowstack<N, 4><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
-                else if (p.lk == 3) tnk::cgemm_rowstack<N, 8><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
-                else tnk::cgemm_rowstack<N, 16><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
-            };
-            if (p.ln == 0) by_k(std::integral_constant<int, 1>{});
-            else if (p.ln == 1) by_k(std::integral_constant<int, 2>{});
-            else by_k(std::integral_constant<int, 4>{});
-        }
+        row_roles(cn, s, p, true);
+        tnk::TcGather g;
+        RC(fill_gather(cn, s, s.nn > s.nm ? 1 : 0, g));
+        const int S = tnk::kTcMaxStack;
+        int *stack = static_cast<int *>(cn.stacks.p);
+        tnk::tc_stack_build<<<1, 1024, (size_t)8 << cn.net.n_beta, st>>>(g, cn.net.n_beta, S, stack);
+        CK(cudaGetLastError());
+        // items of up to 2048 rows; the number of stacks is known on the device only
+        const long long most = (1LL << (s.nbat + p.lm - 8));
+        const unsigned blocks = (unsigned)std::min<long long>(most, 4LL * num_sms());
+        auto by_k = [&](auto n_tag) {
+            constexpr int N = decltype(n_tag)::value;
+            if (p.lk == 2) tnk::cgemm_rowstack<N, 4><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
+            else if (p.lk == 3) tnk::cgemm_rowstack<N, 8><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
+            else tnk::cgemm_rowstack<N, 16><<<blocks, tnk::kRowStackRows, 0, st>>>(p, g, stack, S);
+        };
+        if (p.ln == 0) by_k(std::integral_constant<int, 1>{});
+        else if (p.ln == 1) by_k(std::integral_constant<int, 2>{});
+        else by_k(std::integral_constant<int, 4>{});
     } else if (var == kVarSkinny) {
         if (!skinny_fits(cn, s)) { tn_set_error("long-K kernel: unsupported step shape"); return TN_EINVAL; }
-        if constexpr (sizeof(T) == sizeof(float2)) {
-            const size_t si2 = &s - cn.steps.data();
-            if (cn.cur_closed && skinny_fuses(cn, si2)) {
-                const auto *gd = static_cast<const tnk::GatherDesc *>(cn.gdescs.p) + cn.cp.gd_off[si2];
-                p.gA = s.gat[0] ? gd : nullptr;
-                p.gB = s.gat[1] ? gd + (s.gat[0] ? 1 : 0) : nullptr;
-                p.closed_bits = cn.cur_closed;
-            }
-            // the longer side are the kernel's rows (C = A B^T is symmetric in the roles)
-            if (p.ln > p.lm) {
-                std::swap(p.ptrA, p.ptrB);
-                std::swap(p.gA, p.gB);
-                std::swap(p.lm, p.ln);
-                for (int i = 0; i < tnk::kMaxBits; i++) std::swap(p.pos_m[i], p.pos_n[i]);
-            }
-            // blocks of W warps with MW rows of A each (W MW = min(M, 32) rows per block),
-            // as many as fit at once (each streams its share of the units through its ring)
-            const long long units = (p.nver << p.lbat) * std::max(1, (1 << p.lm) / 32);
-            int rc_go = TN_OK;
-            auto go = [&](auto kern, int warps, int stage_bytes) {
-                const int smem = tnk::kSkinnyST * stage_bytes;
-                int per_sm = 0;
-                if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem) != cudaSuccess ||
-                    per_sm < 1) {
-                    tn_set_error("long-K kernel: launch configuration rejected");
-                    rc_go = TN_EDEVICE;
-                    return;
-                }
-                const unsigned blocks = (unsigned)std::min<long long>(units, (long long)per_sm * num_sms());
-                kern<<<blocks, 32 * warps, smem, st>>>(p);
-            };
-            auto by_n = [&](auto m_tag) {
-                constexpr int M = decltype(m_tag)::value;
-                constexpr int MW = M >= 4 ? 4 : M, W = M / MW;
-                switch (p.ln) {
-                    case 0: go(tnk::cgemm_skinny<W, MW, 1>, W, tnk::skinny_stage_bytes<W, MW, 1>()); break;
-                    case 1: go(tnk::cgemm_skinny<W, MW, 2>, W, tnk::skinny_stage_bytes<W, MW, 2>()); break;
-                    case 2: go(tnk::cgemm_skinny<W, MW, 4>, W, tnk::skinny_stage_bytes<W, MW, 4>()); break;
-                    default: go(tnk::cgemm_skinny<W, MW, 8>, W, tnk::skinny_stage_bytes<W, MW, 8>()); break;
-                }
-            };
-            switch (p.lm) {
-                case 0: by_n(std::integral_constant<int, 1>{}); break;
-                case 1: by_n(std::integral_constant<int, 2>{}); break;
-                case 2: by_n(std::integral_constant<int, 4>{}); break;
-                case 3: by_n(std::integral_constant<int, 8>{}); break;
-                case 4: by_n(std::integral_constant<int, 16>{}); break;
-                default: by_n(std::integral_constant<int, 32>{}); break;  // 64 rows: two row blocks
-            }
-            if (rc_go != TN_OK) return rc_go;
-        } else {
-            tn_set_error("long-K kernel on a complex128 network");
-            return TN_EINVAL;
+        const size_t si2 = &s - cn.steps.data();
+        if (cn.cur_closed && skinny_fuses(cn, si2)) {
+            const auto *gd = static_cast<const tnk::GatherDesc *>(cn.gdescs.p) + cn.cp.gd_off[si2];
+            p.gA = s.gat[0] ? gd : nullptr;
+            p.gB = s.gat[1] ? gd + (s.gat[0] ? 1 : 0) : nullptr;
+            p.closed_bits = cn.cur_closed;
         }
+        // the longer side are the kernel's rows (C = A B^T is symmetric in the roles)
+        if (p.ln > p.lm) {
+            std::swap(p.ptrA, p.ptrB);
+            std::swap(p.gA, p.gB);
+            std::swap(p.lm, p.ln);
+            for (int i = 0; i < tnk::kMaxBits; i++) std::swap(p.pos_m[i], p.pos_n[i]);
+        }
+        // blocks of W warps with MW rows of A each (W MW = min(M, 32) rows per block),
+        // as many as fit at once (each streams its share of the units through its ring)
+        const long long units = (p.nver << p.lbat) * std::max(1, (1 << p.lm) / 32);
+        int rc_go = TN_OK;
+        auto go = [&](auto kern, int warps, int stage_bytes) {
+            const int smem = tnk::kSkinnyST * stage_bytes;
+            int per_sm = 0;
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem) != cudaSuccess ||
+                per_sm < 1) {
+                tn_set_error("long-K kernel: launch configuration rejected");
+                rc_go = TN_EDEVICE;
+                return;
+            }
+            const unsigned blocks = (unsigned)std::min<long long>(units, (long long)per_sm * num_sms());
+            kern<<<blocks, 32 * warps, smem, st>>>(p);
+        };
+        auto by_n = [&](auto m_tag) {
+            constexpr int M = decltype(m_tag)::value;
+            constexpr int MW = M >= 4 ? 4 : M, W = M / MW;
+            switch (p.ln) {
+                case 0: go(tnk::cgemm_skinny<W, MW, 1>, W, tnk::skinny_stage_bytes<W, MW, 1>()); break;
+                case 1: go(tnk::cgemm_skinny<W, MW, 2>, W, tnk::skinny_stage_bytes<W, MW, 2>()); break;
+                case 2: go(tnk::cgemm_skinny<W, MW, 4>, W, tnk::skinny_stage_bytes<W, MW, 4>()); break;
+                default: go(tnk::cgemm_skinny<W, MW, 8>, W, tnk::skinny_stage_bytes<W, MW, 8>()); break;
+            }
+        };
+        switch (p.lm) {
+            case 0: by_n(std::integral_constant<int, 1>{}); break;
+            case 1: by_n(std::integral_constant<int, 2>{}); break;
+            case 2: by_n(std::integral_constant<int, 4>{}); break;
+            case 3: by_n(std::integral_constant<int, 8>{}); break;
+            case 4: by_n(std::integral_constant<int, 16>{}); break;
+            default: by_n(std::integral_constant<int, 32>{}); break;  // 64 rows: two row blocks
+        }
+        if (rc_go != TN_OK) return rc_go;
     } else if (var == kVarRow) {
         row_roles(cn, s, p, row_fuses(cn, si));
         long long rows = p.nver << (p.lbat + p.lm);
         // grid-stride: at most 16 resident blocks' worth per SM, each thread several rows
         unsigned blocks = (unsigned)std::min<long long>((rows + 255) / 256, 16LL * num_sms());
         switch (p.ln) {
-            case 0: tnk::cgemm_row<T, 1><<<blocks, 256, 0, st>>>(p); break;
-            case 1: tnk::cgemm_row<T, 2><<<blocks, 256, 0, st>>>(p); break;
-            case 2: tnk::cgemm_row<T, 4><<<blocks, 256, 0, st>>>(p); break;
-            case 3: tnk::cgemm_row<T, 8><<<blocks, 256, 0, st>>>(p); break;
-            case 4: tnk::cgemm_row<T, 16><<<blocks, 256, 0, st>>>(p); break;
-            default: tnk::cgemm_row<T, 32><<<blocks, 256, 0, st>>>(p); break;
+            case 0: tnk::cgemm_row<float2, 1><<<blocks, 256, 0, st>>>(p); break;
+            case 1: tnk::cgemm_row<float2, 2><<<blocks, 256, 0, st>>>(p); break;
+            case 2: tnk::cgemm_row<float2, 4><<<blocks, 256, 0, st>>>(p); break;
+            case 3: tnk::cgemm_row<float2, 8><<<blocks, 256, 0, st>>>(p); break;
+            case 4: tnk::cgemm_row<float2, 16><<<blocks, 256, 0, st>>>(p); break;
+            default: tnk::cgemm_row<float2, 32><<<blocks, 256, 0, st>>>(p); break;
         }
     } else {
-        if constexpr (sizeof(T) == sizeof(float2)) row_roles(cn, s, p, tile_fuses(cn, si));
+        row_roles(cn, s, p, tile_fuses(cn, si));
         auto launch = [&](auto kern, int TM, int TN, int threads) {
             int ltm = std::min(p.lm, __builtin_ctz(TM)), ltn = std::min(p.ln, __builtin_ctz(TN));
             long long blocks = p.nver << (p.lbat + (p.lm - ltm) + (p.ln - ltn));
             kern<<<(unsigned)blocks, threads, 0, st>>>(p);
         };
         int rc = TN_OK;
-        if constexpr (sizeof(T) == sizeof(float2)) {
-            auto tile = [&](auto sw) {
-                constexpr bool SW = decltype(sw)::value;
-                switch (var) {
-                    case 128064: launch(tnk::cgemm_tile2<128, 64, 8, 8, 8, SW>, 128, 64, 128); break;
-                    case 64064: launch(tnk::cgemm_tile2<64, 64, 4, 8, 8, SW>, 64, 64, 128); break;
-                    case 128032: launch(tnk::cgemm_tile2<128, 32, 8, 4, 8, SW>, 128, 32, 128); break;
-                    case 64032: launch(tnk::cgemm_tile2<64, 32, 4, 4, 8, SW>, 64, 32, 128); break;
-                    case 32032: launch(tnk::cgemm_tile2<32, 32, 4, 2, 8, SW>, 32, 32, 128); break;
-                    case 256016: launch(tnk::cgemm_tile2<256, 16, 8, 4, 8, SW>, 256, 16, 128); break;
-                    case 128016: launch(tnk::cgemm_tile2<128, 16, 4, 4, 8, SW>, 128, 16, 128); break;
-                    case 256008: launch(tnk::cgemm_tile2<256, 8, 8, 2, 8, SW>, 256, 8, 128); break;
-                    case 256004: launch(tnk::cgemm_tile2<256, 4, 4, 2, 8, SW>, 256, 4, 128); break;
-                    case 16016: launch(tnk::cgemm_tile2<16, 16, 4, 2, 8, SW>, 16, 16, 32); break;
-                    default: rc = TN_EINVAL; break;
-                }
-            };
-            if (p.swapped) tile(std::true_type{});
-            else tile(std::false_type{});
-        } else {
+        auto tile = [&](auto sw) {
+            constexpr bool SW = decltype(sw)::value;
             switch (var) {
-                case 128064: launch(tnk::cgemm_tile<T, 128, 64, 8, 8, 4>, 128, 64, 256); break;
-                case 64064: launch(tnk::cgemm_tile<T, 64, 64, 8, 4, 4>, 64, 64, 256); break;
-                case 128032: launch(tnk::cgemm_tile<T, 128, 32, 8, 8, 2>, 128, 32, 256); break;
-                case 64032: launch(tnk::cgemm_tile<T, 64, 32, 8, 4, 2>, 64, 32, 256); break;
-                case 32032: launch(tnk::cgemm_tile<T, 32, 32, 8, 2, 2>, 32, 32, 256); break;
-                case 128016: launch(tnk::cgemm_tile<T, 128, 16, 8, 4, 2>, 128, 16, 256); break;
-                default: launch(tnk::cgemm_tile<T, 16, 16, 8, 1, 1>, 16, 16, 256); break;
+                case 128064: launch(tnk::cgemm_tile<128, 64, 8, 8, 8, SW>, 128, 64, 128); break;
+                case 64064: launch(tnk::cgemm_tile<64, 64, 4, 8, 8, SW>, 64, 64, 128); break;
+                case 128032: launch(tnk::cgemm_tile<128, 32, 8, 4, 8, SW>, 128, 32, 128); break;
+                case 64032: launch(tnk::cgemm_tile<64, 32, 4, 4, 8, SW>, 64, 32, 128); break;
+                case 32032: launch(tnk::cgemm_tile<32, 32, 4, 2, 8, SW>, 32, 32, 128); break;
+                case 256016: launch(tnk::cgemm_tile<256, 16, 8, 4, 8, SW>, 256, 16, 128); break;
+                case 128016: launch(tnk::cgemm_tile<128, 16, 4, 4, 8, SW>, 128, 16, 128); break;
+                case 256008: launch(tnk::cgemm_tile<256, 8, 8, 2, 8, SW>, 256, 8, 128); break;
+                case 256004: launch(tnk::cgemm_tile<256, 4, 4, 2, 8, SW>, 256, 4, 128); break;
+                case 16016: launch(tnk::cgemm_tile<16, 16, 4, 2, 8, SW>, 16, 16, 32); break;
+                default: rc = TN_EINVAL; break;
             }
-        }
+        };
+        if (p.swapped) tile(std::true_type{});
+        else tile(std::false_type{});
         if (rc != TN_OK) { tn_set_error("unknown kernel variant " + std::to_string(var)); return rc; }
     }
     CK(cudaGetLastError());
     return TN_OK;
 }
 
-template <typename T>
 int launch_step(CNet &cn, const Step &s, cudaStream_t st) {
     const size_t si = &s - cn.steps.data();
     const int var = si < cn.variant.size() && cn.variant[si] >= 0 ? cn.variant[si] : default_variant(cn, si);
-    return launch_variant<T>(cn, s, st, var);
+    return launch_variant(cn, s, st, var);
 }
 
 int launch_gathers(CNet &cn, size_t si, const uint64_t *d_closed, cudaStream_t st) {
@@ -1235,8 +1207,7 @@ int launch_slice_sum(CNet &cn, double2 *out, cudaStream_t st) {
         }
         CK(cudaEventRecord(cn.ev[2 * ss], st));
     }
-    if (cn.elem == 8) tnk::slice_sum<float2><<<blocks, 256, 0, st>>>(rt, cn.cp.root_nver, nfree, nout, out);
-    else tnk::slice_sum<double2><<<blocks, 256, 0, st>>>(rt, cn.cp.root_nver, nfree, nout, out);
+    tnk::slice_sum<float2><<<blocks, 256, 0, st>>>(rt, cn.cp.root_nver, nfree, nout, out);
     CK(cudaGetLastError());
     if (cn.trace) {
         CK(cudaEventRecord(cn.ev[2 * ss + 1], st));
@@ -1428,8 +1399,9 @@ int launch_root_slice_sum(CNet &cn, size_t si, double2 *out, cudaStream_t st) {
         if (p.lk == 0) tnk::root_sum_small<0><<<blocks, 256, smem, st>>>(p, nfree, nout, out);
         else if (p.lk == 1) tnk::root_sum_small<1><<<blocks, 256, smem, st>>>(p, nfree, nout, out);
         else tnk::root_sum_small<2><<<blocks, 256, smem, st>>>(p, nfree, nout, out);
-    } else if (cn.elem == 8) tnk::root_slice_sum<float2><<<blocks, 256, 0, st>>>(p, nfree, nout, out);
-    else tnk::root_slice_sum<double2><<<blocks, 256, 0, st>>>(p, nfree, nout, out);
+    } else {
+        tnk::root_slice_sum<float2><<<blocks, 256, 0, st>>>(p, nfree, nout, out);
+    }
     CK(cudaGetLastError());
     if (cn.trace) {
         CK(cudaEventRecord(cn.ev[2 * ss + 1], st));
@@ -1486,8 +1458,7 @@ int execute(CNet &cn, const uint64_t *d_closed, bool skip_beta_free, double2 *ou
         const int var = si < cn.variant.size() && cn.variant[si] >= 0 ? cn.variant[si] : default_variant(cn, si);
         const bool in_place = d_closed && reads_in_place(cn, si, var);
         if (!in_place) RC(launch_gathers(cn, si, d_closed, st));
-        if (cn.elem == 8) RC(launch_step<float2>(cn, s, st));
-        else RC(launch_step<double2>(cn, s, st));
+        RC(launch_step(cn, s, st));
         if (cn.calibrating) {
             const long long n = 1LL << cn.tree.nodes[s.c].layout.size();
             for (long long v = 0; v < cn.cp.nver[s.c]; v++) {
@@ -1558,7 +1529,6 @@ bool resolve_variants(CNet &cn) {
 // One full execution that times each applicable variant of every step still unchosen
 // (one warm-up launch, then two timed launches, CUDA events on the plan's stream),
 // keeps the fastest and then runs it, so `out` is written as by execute().
-template <typename T>
 int tune_execute(CNet &cn, const uint64_t *d_closed, double2 *out, cudaStream_t st) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
@@ -1576,9 +1546,9 @@ int tune_execute(CNet &cn, const uint64_t *d_closed, double2 *out, cudaStream_t 
             int best = -1;
             float best_ms = 0;
             for (int v : step_variants(cn, si)) {
-                rc = launch_variant<T>(cn, s, st, v);
+                rc = launch_variant(cn, s, st, v);
                 if (rc == TN_OK && cudaEventRecord(e0, st) != cudaSuccess) rc = TN_EDEVICE;
-                for (int r = 0; r < 2 && rc == TN_OK; r++) rc = launch_variant<T>(cn, s, st, v);
+                for (int r = 0; r < 2 && rc == TN_OK; r++) rc = launch_variant(cn, s, st, v);
                 float ms = 0;
                 if (rc == TN_OK && (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
                                     cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)) {
@@ -1594,7 +1564,7 @@ int tune_execute(CNet &cn, const uint64_t *d_closed, double2 *out, cudaStream_t 
                 g_tune[tune_key(cn, si)] = best;
             }
         }
-        if (rc == TN_OK) rc = launch_step<T>(cn, s, st);
+        if (rc == TN_OK) rc = launch_step(cn, s, st);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1653,7 +1623,7 @@ int execute_graphed(DevMem &mem, CNet &cn, const uint64_t *d_closed, bool skip_b
     }
     if (resolve_variants(cn)) {
         drop_graphs(cn);
-        return cn.elem == 8 ? tune_execute<float2>(cn, d_closed, out, st) : tune_execute<double2>(cn, d_closed, out, st);
+        return tune_execute(cn, d_closed, out, st);
     }
     static const bool disabled = getenv("TN_NO_GRAPH") != nullptr;
     if (cn.trace || disabled) return execute(cn, d_closed, skip_beta_free, out, st);
@@ -2208,7 +2178,8 @@ int tn_spoof(tn_plan_h p, const uint64_t *slices, int64_t n_slices, uint64_t clo
     CK(cudaMemcpyAsync(p->d_closed.p, &closed_pattern, sizeof(uint64_t), cudaMemcpyHostToDevice, st));
     RC(execute_graphed(p->mem, p->amp, static_cast<const uint64_t *>(p->d_closed.p), false,
                        static_cast<double2 *>(p->d_amps.p), st, p->budget));
-    if (M > tnk::kSelCluster * tnk::kSelBlock * tnk::kSelKeys) { tn_set_error("tn_spoof: batch too large"); return TN_EUNSUPPORTED; }
+    // tn_plan allows 16 open qubits, 2^16 strings: what one cluster holds
+    static_assert(tnk::kSelCluster * tnk::kSelBlock * tnk::kSelKeys >= 1 << 16, "spoof_select holds a batch");
     RC(ensure(p->mem, p->d_sbits, N * sizeof(unsigned long long)));
     if (probs) RC(ensure(p->mem, p->d_sprob, N * sizeof(double)));
     unsigned long long base = 0;

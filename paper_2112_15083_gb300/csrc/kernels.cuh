@@ -132,9 +132,6 @@ template <typename T> __device__ __forceinline__ void store_c_t(const GemmParams
 template <> __device__ __forceinline__ void store_c_t<float2>(const GemmParams &p, long long v, long long off, float2 x) {
     store_c(p, v, off, x);
 }
-template <> __device__ __forceinline__ void store_c_t<double2>(const GemmParams &p, long long v, long long off, double2 x) {
-    static_cast<double2 *>(p.C)[v * p.c_vstride + off] = x;
-}
 
 __device__ __forceinline__ long long scatter_bits(long long x, const int8_t *pos, int nbits) {
     long long off = 0;
@@ -150,16 +147,8 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
     c.y = fmaf(a.y, b.x, c.y);
     return c;
 }
-__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {
-    c.x = fma(a.x, b.x, c.x);
-    c.x = fma(-a.y, b.y, c.x);
-    c.y = fma(a.x, b.y, c.y);
-    c.y = fma(a.y, b.x, c.y);
-    return c;
-}
 template <typename T> __device__ __forceinline__ T czero();
 template <> __device__ __forceinline__ float2 czero<float2>() { return make_float2(0.f, 0.f); }
-template <> __device__ __forceinline__ double2 czero<double2>() { return make_double2(0.0, 0.0); }
 
 // One output row (v, bat, m) per thread and call; all N (<= 32) columns in registers.  For the
 // gate-absorption steps (small N and K), which are bound by HBM bandwidth.
@@ -728,77 +717,6 @@ __global__ void __launch_bounds__(256) cgemm_small(GemmParams p, SmallMap smp) {
     }
 }
 
-// Shared-memory tiled kernel: TM x TN output tile, K in chunks of TK, each thread an
-// RM x RN register tile (rows contiguous, columns strided by TN/RN for coalescing).
-template <typename T, int TM, int TN, int TK, int RM, int RN>
-__global__ void __launch_bounds__((TM / RM) * (TN / RN)) cgemm_tile(GemmParams p) {
-    constexpr int NTX = TN / RN, NTY = TM / RM, NT = NTX * NTY;
-    __shared__ T As[TK][TM + 1];
-    __shared__ T Bs[TK][TN + 1];
-    const int tid = threadIdx.x;
-    const int tx = tid % NTX, ty = tid / NTX;
-    const long long M = 1LL << p.lm, N = 1LL << p.ln;
-    const int K = 1 << p.lk;
-    const int ltm = p.lm > 0 ? min(p.lm, __ffs(TM) - 1) : 0;
-    const int ltn = p.ln > 0 ? min(p.ln, __ffs(TN) - 1) : 0;
-    const int ltiles_m = p.lm - ltm, ltiles_n = p.ln - ltn;
-    long long bid = blockIdx.x;
-    const long long tn_i = bid & ((1LL << ltiles_n) - 1);
-    bid >>= ltiles_n;
-    const long long tm_i = bid & ((1LL << ltiles_m) - 1);
-    bid >>= ltiles_m;
-    const long long bat = bid & ((1LL << p.lbat) - 1);
-    const long long v = bid >> p.lbat;
-    if (v >= p.nver) return;
-    const long long m0 = tm_i * TM, n0 = tn_i * TN;
-    const int mrows = (int)min((long long)TM, M - m0), ncols = (int)min((long long)TN, N - n0);
-    const T *A = static_cast<const T *>(p.ptrA[v]) + (((bat << p.lm) | m0) << p.lk);
-    const T *B = static_cast<const T *>(p.ptrB[v]) + (((bat << p.ln) | n0) << p.lk);
-    T acc[RM][RN];
-#pragma unroll
-    for (int i = 0; i < RM; i++)
-#pragma unroll
-        for (int j = 0; j < RN; j++) acc[i][j] = czero<T>();
-    const int kt = min(TK, K);
-    const int lkt = __ffs(kt) - 1;
-    for (int k0 = 0; k0 < K; k0 += kt) {
-        for (int e = tid; e < (TM << lkt); e += NT) {
-            int r = e >> lkt, c = e & (kt - 1);
-            As[c][r] = r < mrows ? A[((long long)r << p.lk) + k0 + c] : czero<T>();
-        }
-        for (int e = tid; e < (TN << lkt); e += NT) {
-            int r = e >> lkt, c = e & (kt - 1);
-            Bs[c][r] = r < ncols ? B[((long long)r << p.lk) + k0 + c] : czero<T>();
-        }
-        __syncthreads();
-        for (int kk = 0; kk < kt; kk++) {
-            T a[RM], b[RN];
-#pragma unroll
-            for (int i = 0; i < RM; i++) a[i] = As[kk][ty * RM + i];
-#pragma unroll
-            for (int j = 0; j < RN; j++) b[j] = Bs[kk][tx + j * NTX];
-#pragma unroll
-            for (int i = 0; i < RM; i++)
-#pragma unroll
-                for (int j = 0; j < RN; j++) acc[i][j] = cfma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    const long long cb = scatter_bits(bat, p.pos_bat, p.lbat);
-    long long offn[RN];
-#pragma unroll
-    for (int j = 0; j < RN; j++) offn[j] = scatter_bits(n0 + tx + j * NTX, p.pos_n, p.ln);
-#pragma unroll
-    for (int i = 0; i < RM; i++) {
-        const int r = ty * RM + i;
-        if (r >= mrows) continue;
-        const long long offm = cb + scatter_bits(m0 + r, p.pos_m, p.lm);
-#pragma unroll
-        for (int j = 0; j < RN; j++)
-            if (tx + j * NTX < ncols) store_c_t<T>(p, v, offm + offn[j], acc[i][j]);
-    }
-}
-
 // Packed FP32 multiply-add: two independent fmaf in one instruction.
 __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
     unsigned long long d;
@@ -836,7 +754,7 @@ __device__ __forceinline__ float2 unpack2(unsigned long long x) {
 // buffers; the next chunk's loads are in flight during the products.  Gathered operands
 // whose batch block is contiguous in the stored form are read in place.
 template <int TM, int TN, int RM, int RN, int TK, bool SW>
-__global__ void __launch_bounds__((TM / RM) * (TN / RN)) cgemm_tile2(GemmParams p) {
+__global__ void __launch_bounds__((TM / RM) * (TN / RN)) cgemm_tile(GemmParams p) {
     constexpr int NTX = TN / RN, NTY = TM / RM, NT = NTX * NTY, GM = RM / 4, GN = RN / 2;
     constexpr int LA = (TM * TK / 2 + NT - 1) / NT, LB = (TN * TK / 2 + NT - 1) / NT;
     static_assert(TM <= NT * LA && TN <= NT * LB, "K = 1 loads one element per slot");
@@ -1018,7 +936,7 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN)) cgemm_tile2(GemmParams 
 struct MatDesc {
     const double2 *src;  // full leaf tensor, data index = sum_t value(leg t) << t
     void *dst;           // [code][2^nd] in the consumer's layout and format
-    int fmt;             // OutFmt (complex64 leaves only; complex128 when T = double2)
+    int fmt;             // OutFmt
     float scale;         // multiplier (split fp16 range scaling)
     int nd;              // destination bits
     int ncode_bits;      // sliced legs of the leaf
@@ -1027,7 +945,6 @@ struct MatDesc {
 };
 
 // grid.y = leaf; threads over (code, element).
-template <typename T>
 __global__ void materialize(const MatDesc *descs) {
     const MatDesc d = descs[blockIdx.y];
     const long long total = 1LL << (d.nd + d.ncode_bits);
@@ -1038,17 +955,13 @@ __global__ void materialize(const MatDesc *descs) {
         for (int t = 0; t < d.nd; t++) src |= ((e >> t) & 1) << d.dst_leg[t];
         for (int u = 0; u < d.ncode_bits; u++) src |= ((code >> u) & 1) << d.sl_leg[u];
         const double2 x = d.src[src];
-        if constexpr (sizeof(T) == sizeof(float2)) {
-            const float2 y = make_float2((float)(x.x * d.scale), (float)(x.y * d.scale));
-            if (d.fmt == OUT_C64) {
-                static_cast<float2 *>(d.dst)[g] = y;
-            } else {
-                const long long ne = 1LL << d.nd;
-                unsigned short *base = static_cast<unsigned short *>(d.dst) + 4 * code * ne;
-                store_split(base, ne, e, y, d.fmt == OUT_SPLIT_FP16);
-            }
+        const float2 y = make_float2((float)(x.x * d.scale), (float)(x.y * d.scale));
+        if (d.fmt == OUT_C64) {
+            static_cast<float2 *>(d.dst)[g] = y;
         } else {
-            static_cast<T *>(d.dst)[g] = x;
+            const long long ne = 1LL << d.nd;
+            unsigned short *base = static_cast<unsigned short *>(d.dst) + 4 * code * ne;
+            store_split(base, ne, e, y, d.fmt == OUT_SPLIT_FP16);
         }
     }
 }
@@ -1123,7 +1036,6 @@ __global__ void absmax_kernel(const void *data, long long n, int fmt, int *absma
 // complex64 inputs are widened with integer operations (exact), which leaves the FP64
 // pipe to the additions.
 __device__ __forceinline__ double slice_widen(float x) { return tn_widen(x); }
-__device__ __forceinline__ double slice_widen(double x) { return x; }
 
 template <typename T>
 __global__ void slice_sum(const void *const *ptr, long long nver, int nfree, int nout, double2 *out) {
@@ -1217,14 +1129,12 @@ __device__ __forceinline__ T root_value(const GemmParams &p, long long v, long l
     return acc;
 }
 
-// What store_c_t applies before storing: the output scale for complex64, nothing for
-// complex128.
+// What store_c_t applies before storing: the output scale.
 __device__ __forceinline__ float2 root_scaled(const GemmParams &p, float2 x) {
     x.x *= p.out_scale;
     x.y *= p.out_scale;
     return x;
 }
-__device__ __forceinline__ double2 root_scaled(const GemmParams &, double2 x) { return x; }
 
 constexpr int kRootTabBytes = 3;  // free patterns of up to 24 bits
 
