@@ -347,6 +347,15 @@ def launches_per(s):
     return 1 + s["gathers"] + (1 if s["kernel"] in STACKED_VARIANTS or s["kernel"] == 6 else 0)
 
 
+def replayed_launches(plan, groups, traced):
+    """Kernel launches of `groups` batch groups as they are replayed, the first with every
+    step and the later ones reusing the stem; `traced`, their count when every step is a
+    launch of its own, where the plan has replayed none."""
+    count = getattr(plan, "replayed_launches", lambda reuse: 0)
+    first, later = count(False), count(True)
+    return first + (groups - 1) * later if first and (later or groups == 1) else traced
+
+
 def kernel_name(k):
     if k in STACKED_VARIANTS:
         return "tc_cgemm<%d,%d> stacked" % (k - 19000, {19128: 3, 19064: 4}[k])
@@ -582,8 +591,8 @@ def run_group(args, with_e2e=True, with_cpu=True):
         "cpu_baseline": cpu, "e2e": e2e, "top_steps": top_steps_of(steps_tr), "slice_sum": slice_sum_of(ssum),
         # the job's contraction launches, batch gathers and slice sums, plus a batch draw and
         # a sampler launch per step
-        "gpu_launches": (sum(s["launches"] * launches_per(s) for s in steps_tr)
-                         + sum(s["launches"] for s in ssum) + 2 * args.steps),
+        "gpu_launches": replayed_launches(plan, args.steps, sum(s["launches"] * launches_per(s) for s in steps_tr)
+                                          + sum(s["launches"] for s in ssum)) + 2 * args.steps,
     }
 
 
@@ -702,7 +711,7 @@ def run_job(args):
     plan.trace(False)
     steps_tr, ssum = split_trace(trace)
     # launch gaps: the graph-replayed chunk against the sum of its launches' device times
-    # (the traced chunk runs the same launches one by one, CUDA events around each); the
+    # (the traced chunk runs every step as a launch of its own, CUDA events around each); the
     # difference also holds the per-group pattern copies and FP64 accumulations
     launches_ms = sum(s["ms"] for s in steps_tr) + sum(s["ms"] for s in ssum)
     gaps = {"chunk_ms_replayed": round(tot_ms / args.steps, 2), "launch_device_ms_sum": round(launches_ms, 2),
@@ -747,8 +756,8 @@ def run_job(args):
 
     if rank != 0:
         return None
-    per_chunk_launches = (sum(s["launches"] * launches_per(s) for s in steps_tr) + sum(s["launches"] for s in ssum)
-                          + info["groups"])
+    per_chunk_launches = info["groups"] + replayed_launches(
+        plan, info["groups"], sum(s["launches"] * launches_per(s) for s in steps_tr) + sum(s["launches"] for s in ssum))
     return {
         "metric": METRIC, "value": value, "unit": "samples/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": tot_ms / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -767,7 +776,7 @@ def run_job(args):
         "cpu_baseline": cpu, "e2e": e2e, "top_steps": top_steps_of(steps_tr, 8), "slice_sum": slice_sum_of(ssum),
         "secondary": secondary, "launch_gaps": gaps,
         # per chunk: every contraction launch, its gathers and slice sums, one amplitude
-        # accumulation per group (counted from the traced chunk)
+        # accumulation per group
         "gpu_launches": per_chunk_launches * args.steps,
     }
 

@@ -391,8 +391,14 @@ int tn_sample_step(tn_plan_h p, const uint64_t *slices, int64_t n_slices, double
  */
 int tn_plan_test_stall(tn_plan_h p, int64_t cycles);
 
+/* Kernel launches of one execution as it is replayed (small steps share launches, the slice
+ * sum may run with the root step), of every step (reuse_stem = 0) or of a later batch group
+ * (1): those of the replay captured last, 0 before the first. */
+int tn_plan_launches(tn_plan_h p, int32_t reuse_stem, int32_t *n_launches);
+
 /* Tracing: when on, every execution records CUDA events around each contraction step
- * and around the FP64 slice sum on the plan's stream.  tn_trace_read synchronises and
+ * and around the FP64 slice sum on the plan's stream.  A traced execution launches every step
+ * by itself, also those that share a launch in a replay.  tn_trace_read synchronises and
  * reports, per step, the launches, the summed device time, and the algorithmic FLOPs
  * (8 per complex multiply-add) and bytes (operands read + result written, complex64) of
  * one launch; entry n_steps (the last) is the slice sum (FLOPs = FP64 additions). */

@@ -165,6 +165,7 @@ struct CNet {
     // call plan and the (closed-pattern, output) buffers they were captured with
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     const void *graph_key[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    int graph_kernels[2] = {0, 0};  // kernel launches of the execution captured last (tn_plan_launches)
     int elem = 8;  // bytes per element (complex64, or four 16-bit planes)
     std::vector<DBuf> leaf_src, leaf_dst;
     std::vector<int> leaf_codebits;
@@ -1613,6 +1614,20 @@ cudaStream_t capture_stream() {
     return s;
 }
 
+int count_kernels(cudaGraph_t g, int &n) {
+    size_t n_nodes = 0;
+    CK(cudaGraphGetNodes(g, nullptr, &n_nodes));
+    std::vector<cudaGraphNode_t> nodes(n_nodes);
+    CK(cudaGraphGetNodes(g, nodes.data(), &n_nodes));
+    n = 0;
+    for (cudaGraphNode_t x : nodes) {
+        cudaGraphNodeType t;
+        CK(cudaGraphNodeGetType(x, &t));
+        n += t == cudaGraphNodeTypeKernel;
+    }
+    return TN_OK;
+}
+
 // execute() through a CUDA graph: the first execution for a (call plan, buffers, stem
 // mode) is captured on an internal stream, later ones replay the graph on `st`.
 int execute_graphed(DevMem &mem, CNet &cn, const uint64_t *d_closed, bool skip_beta_free, double2 *out,
@@ -1646,6 +1661,10 @@ int execute_graphed(DevMem &mem, CNet &cn, const uint64_t *d_closed, bool skip_b
         if (ec != cudaSuccess || !g) {
             tn_set_error(std::string("graph capture failed: ") + cudaGetErrorString(ec));
             return TN_EDEVICE;
+        }
+        if ((rc = count_kernels(g, cn.graph_kernels[gi])) != TN_OK) {
+            cudaGraphDestroy(g);
+            return rc;
         }
         cudaError_t ei = cudaGraphInstantiate(&cn.graph[gi], g, 0);
         cudaGraphDestroy(g);
@@ -2380,6 +2399,12 @@ int tn_plan_sync(tn_plan_h p) {
     if (!p) { tn_set_error("null plan"); return TN_EINVAL; }
     CK(cudaStreamSynchronize(p->mem.stream));
     return check_err(p->amp, p->mem.stream);
+}
+
+int tn_plan_launches(tn_plan_h p, int32_t reuse_stem, int32_t *n_launches) {
+    if (!p || !n_launches) { tn_set_error("null argument"); return TN_EINVAL; }
+    *n_launches = p->amp.graph_kernels[reuse_stem ? 1 : 0];
+    return TN_OK;
 }
 
 int tn_trace_enable(tn_plan_h p, int32_t on) {

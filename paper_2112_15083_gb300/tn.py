@@ -23,7 +23,7 @@ EXPORTED = [
     "tn_plan_opts_default", "tn_circuit_load", "tn_circuit_destroy", "tn_plan", "tn_plan_destroy",
     "tn_plan_get_info", "tn_plan_sliced_edges", "tn_partial_norms", "tn_slice_cut", "tn_select",
     "tn_contract", "tn_xeb", "tn_spoof", "tn_sample", "tn_rejection_sample", "tn_draw_batches", "tn_strerror", "tn_last_error",
-    "tn_plan_host", "tn_sliced_vertex_select", "tn_sample_step", "tn_trace_enable", "tn_trace_read",
+    "tn_plan_host", "tn_sliced_vertex_select", "tn_sample_step", "tn_trace_enable", "tn_trace_read", "tn_plan_launches",
     "tn_slice_cut_noalloc", "tn_plan_estimate", "tn_plan_sync", "tn_server_opts_default", "tn_server_create",
     "tn_server_submit", "tn_server_query", "tn_server_wait", "tn_server_get_stats", "tn_server_destroy",
     "tn_plan_test_stall", "tn_job_create", "tn_job_run", "tn_job_get_info", "tn_job_amplitudes", "tn_job_finish", "tn_job_destroy",
@@ -163,6 +163,7 @@ def lib():
         L.tn_sliced_vertex_select.argtypes = [vp, vp, i32, i32, vp, ctypes.POINTER(i32)]
         L.tn_sample_step.argtypes = [vp, vp, i64, dbl, u64, u64, dbl, i32, vp, vp, i32]
         L.tn_trace_enable.argtypes = [vp, i32]
+        L.tn_plan_launches.argtypes = [vp, i32, ctypes.POINTER(i32)]
         L.tn_trace_read.argtypes = [vp, ctypes.POINTER(StepTrace), i32, ctypes.POINTER(i32)]
         L.tn_plan_estimate.argtypes = [vp, vp, i64, ctypes.POINTER(i64), ctypes.POINTER(dbl), ctypes.POINTER(dbl)]
         L.tn_plan_sync.argtypes = [vp]
@@ -429,6 +430,12 @@ class Plan:
         _check(lib().tn_plan_estimate(self.h, _np_ptr(sl), sl.size, ctypes.byref(b), ctypes.byref(f1), ctypes.byref(f2)),
                "tn_plan_estimate")
         return b.value, f1.value, f2.value
+
+    def replayed_launches(self, reuse_stem: bool = False) -> int:
+        """Kernel launches of one replayed execution (tn_plan_launches); 0 before the first."""
+        n = ctypes.c_int32()
+        _check(lib().tn_plan_launches(self.h, int(reuse_stem), ctypes.byref(n)), "tn_plan_launches")
+        return n.value
 
     def trace(self, on: bool = True):
         _check(lib().tn_trace_enable(self.h, int(on)), "tn_trace_enable")
