@@ -194,9 +194,9 @@ int tn_partial_norms(tn_plan_h p, double f, int32_t *s_index, int32_t *k, double
  * Slice cut (Alg. 1 steps 4-5) on the GPU: sort R descending (ties: index ascending),
  * sum in that order in FP64, keep the minimal prefix whose sum reaches f (all of it if
  * rounding keeps the total below f).  R: host array of 2^k doubles.  X: out, host,
- * the kept indices in sorted order (cap 2^k); F: the kept sum.  k <= 12 (one block sorts
- * the 2^k norms in shared memory); larger k returns TN_EINVAL.  The device scratch is
- * allocated and freed on the stream inside the call, which synchronises the stream.
+ * the kept indices in sorted order (cap 2^k); F: the kept sum.  k <= 12 (a block holds
+ * the 2^k norms in shared memory); larger k returns TN_EINVAL.  The call waits for the
+ * stream; its device scratch is allocated on the stream and freed on it at the end.
  */
 int tn_slice_cut(const double *R, int32_t k, double f, void *stream, int32_t *X,
                  int32_t *n_x, double *F);

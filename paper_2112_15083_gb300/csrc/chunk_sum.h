@@ -21,7 +21,7 @@
 //
 // With what is left of lo added in rounded FP32 instead, ahead of the larger parts, a small
 // residual of values that cancel was lost; 20 qubits in split bf16, whose chunks all take the
-// four splits, took 206 us a call so and take 213 us now; 24 qubits in split fp16 879 and 868 us.
+// four splits, took 206 us a call so and take 215 us now; 24 qubits in split fp16 880 and 868 us.
 #pragma once
 
 #include <math.h>

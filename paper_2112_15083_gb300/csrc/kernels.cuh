@@ -90,8 +90,8 @@ struct GemmParams {
     float out_scale;          // multiplier applied before storing
     int swapped;              // operands exchanged (A holds the step's B): keep the step's
                               // operand order inside each complex multiply-add
-    // row kernel only: operands read through their batch gather instead of a gathered
-    // copy (null: not gathered); closed_bits are the group's batch patterns
+    // row, tile, long-K and small-step kernels: operands read through their batch gather
+    // instead of a gathered copy (null: not gathered); closed_bits are the group's patterns
     const GatherDesc *gA, *gB;
     const uint64_t *closed_bits;
     int *err;                 // long-K kernel: set to 1 if a bounded wait gives up
@@ -1734,7 +1734,7 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
 // FP64 comparison of a warp holds the SM's FP64 pipe 16 cycles) took most of 105 us at 2^12 norms:
 // 78 dependent stages on one SM.  The FP64 prefix is a chain of one addition per norm up to
 // the cut; every lane of a warp forms it, lane l keeps the l-th of 32 sums, and the 32
-// comparisons with f are one ballot.  A whole call at 2^12 norms and f = 0.3: 150 -> 75 us.
+// comparisons with f are one ballot.  Repeated whole calls at 2^12 norms and f = 0.3: 150 -> 75 us.
 constexpr int kRankWarps = 8;
 __global__ void __launch_bounds__(32 * kRankWarps) slice_rank(const double *R, int k, int32_t *rank) {
     extern __shared__ unsigned long long rank_key[];
