@@ -174,3 +174,48 @@ inline void layout_call(const Tree &tree, const std::vector<Step> &steps, uint64
     place_call(tree, steps, E, elem, true, L);
     if (L.arena_bytes > least + kSmallBytes) place_call(tree, steps, E, elem, false, L);
 }
+
+// The launches of an execution, in order: each a group of small steps that run together
+// (shared), or one step by itself.
+struct LaunchItem {
+    std::vector<int> steps;
+    bool shared;
+};
+
+// The launch order with the small steps grouped (small: the steps that may be, a subset of
+// L.small); skip_stem: without the batch-independent steps.  Every small step whose operands
+// exist runs in the next shared launch, and when none is ready the next other step follows.
+// The other steps keep their order and a small step never runs later than its place in it, so
+// the arena's reuse (planned in step order) holds; the small steps' own results are never
+// reused.
+inline std::vector<LaunchItem> launch_order(const Tree &tree, const std::vector<Step> &steps, const std::vector<char> &small,
+                                            const std::vector<long long> &nver, bool skip_stem) {
+    std::vector<LaunchItem> out;
+    std::vector<char> done(tree.nodes.size(), 1);
+    std::vector<int> todo;
+    for (size_t i = 0; i < steps.size(); i++)
+        if (!skip_stem || tree.nodes[steps[i].c].beta) todo.push_back((int)i);
+    for (int i : todo) done[steps[i].c] = 0;
+    // one ready step alone shares a launch too if it is tiny (it may join a chain) or would need a
+    // gather launch
+    auto alone = [&](int i) {
+        const Step &s = steps[i];
+        return s.gat[0] || s.gat[1] || (nver[s.c] << (s.nbat + s.nm + s.nn)) <= kSmallAlone;
+    };
+    while (!todo.empty()) {
+        std::vector<int> ready, rest;
+        for (int i : todo) {
+            const Step &s = steps[i];
+            (small[i] && done[s.a] && done[s.b] ? ready : rest).push_back(i);
+        }
+        const bool shared = ready.size() > 1 || (ready.size() == 1 && alone(ready[0]));
+        if (ready.empty()) {
+            ready.push_back(rest[0]);
+            rest.erase(rest.begin());
+        }
+        for (int i : ready) done[steps[i].c] = 1;
+        out.push_back({ready, shared});
+        todo.swap(rest);
+    }
+    return out;
+}

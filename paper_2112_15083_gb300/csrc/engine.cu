@@ -1249,12 +1249,8 @@ bool root_faster(const CNet &cn, size_t si) {
     return (nout <= 18 && products <= 32) || (nout >= 16 && nout <= 20 && terms >= 12);
 }
 
-// The launch order with the small steps grouped: every small step whose operands exist runs in
-// the next small launch, and when none is ready the next other step follows.  The other
-// steps keep their order and a small step never runs later than its place in it, so the
-// arena's reuse (planned in step order) holds; the small steps' own results are never
-// reused.  Steps on the tensor cores, and the root (it may run fused with the slice sum), are
-// not grouped.
+// The launches of an execution (launch_order) with the small steps grouped.  Steps on the tensor
+// cores, and the root (it may run fused with the slice sum), are not grouped.
 int schedule_small(DevMem &mem, CNet &cn) {
     CallPlan &cp = cn.cp;
     const size_t ns = cn.steps.size();
@@ -1271,60 +1267,37 @@ int schedule_small(DevMem &mem, CNet &cn) {
     cp.small_off.assign(1, 0);
     cp.small_run.clear();
     for (int skip = 0; skip < 2; skip++) {
-        std::vector<char> done(cn.tree.nodes.size(), 0);
-        std::vector<int> todo;
-        for (size_t i = 0; i < ns; i++)
-            if (!skip || cn.tree.nodes[cn.steps[i].c].beta) todo.push_back((int)i);
-        for (size_t x = 0; x < done.size(); x++) done[x] = 1;
-        for (int i : todo) done[cn.steps[i].c] = 0;
         std::vector<int> &out = cp.sched[skip];
         out.clear();
         bool chain = false;  // the last item is a run of levels that fit a chain
-        while (!todo.empty()) {
-            std::vector<int> ready, rest;
-            for (int i : todo) {
-                const Step &s = cn.steps[i];
-                (cp.small[i] && done[s.a] && done[s.b] ? ready : rest).push_back(i);
+        for (const LaunchItem &item : launch_order(cn.tree, cn.steps, cp.small, cp.nver, skip != 0)) {
+            if (!item.shared) {
+                out.push_back(item.steps[0]);
+                continue;
             }
-            // one ready step alone: a small launch too if it is tiny (it may join a chain) or would
-            // need a gather launch
-            auto alone = [&](int i) {
+            for (int i : item.steps) {
                 const Step &s = cn.steps[i];
-                return cp.gd_off[i + 1] > cp.gd_off[i] || (cp.nver[s.c] << (s.nbat + s.nm + s.nn)) <= kSmallAlone;
-            };
-            if (ready.size() > 1 || (ready.size() == 1 && alone(ready[0]))) {
-                for (int i : ready) {
-                    const Step &s = cn.steps[i];
-                    tnk::GemmParams p;
-                    RC(step_params(cn, s, p));
-                    const auto *gd = static_cast<const tnk::GatherDesc *>(cn.gdescs.p) + cp.gd_off[i];
-                    p.gA = s.gat[0] ? gd : nullptr;
-                    p.gB = s.gat[1] ? gd + (s.gat[0] ? 1 : 0) : nullptr;
-                    const long long total = p.nver << (p.lbat + p.lm + p.ln);
-                    for (long long o = 0; o < total; o += tnk::kSmallBlock)
-                        blocks.push_back(make_int2((int)descs.size(), (int)o));
-                    descs.push_back(p);
-                }
-                // a level that fits a chain joins the chain of the level just before it
-                const int l = (int)cp.small_off.size() - 1, nb = (int)blocks.size() - cp.small_off[l];
-                cp.small_off.push_back((int)blocks.size());
-                const bool fits = nb <= tnk::kChainBlocks;
-                if (fits && chain && !out.empty() && out.back() < 0) {
-                    cp.small_run.back()[1]++;
-                } else {
-                    cp.small_run.push_back({l, 1});
-                    out.push_back(-(int)cp.small_run.size());
-                }
-                chain = fits;
-            } else if (ready.size() == 1) {
-                out.push_back(ready[0]);
+                tnk::GemmParams p;
+                RC(step_params(cn, s, p));
+                const auto *gd = static_cast<const tnk::GatherDesc *>(cn.gdescs.p) + cp.gd_off[i];
+                p.gA = s.gat[0] ? gd : nullptr;
+                p.gB = s.gat[1] ? gd + (s.gat[0] ? 1 : 0) : nullptr;
+                const long long total = p.nver << (p.lbat + p.lm + p.ln);
+                for (long long o = 0; o < total; o += tnk::kSmallBlock)
+                    blocks.push_back(make_int2((int)descs.size(), (int)o));
+                descs.push_back(p);
+            }
+            // a level that fits a chain joins the chain of the level just before it
+            const int l = (int)cp.small_off.size() - 1, nb = (int)blocks.size() - cp.small_off[l];
+            cp.small_off.push_back((int)blocks.size());
+            const bool fits = nb <= tnk::kChainBlocks;
+            if (fits && chain && !out.empty() && out.back() < 0) {
+                cp.small_run.back()[1]++;
             } else {
-                ready.push_back(rest[0]);
-                out.push_back(rest[0]);
-                rest.erase(rest.begin());
+                cp.small_run.push_back({l, 1});
+                out.push_back(-(int)cp.small_run.size());
             }
-            for (int i : ready) done[cn.steps[i].c] = 1;
-            todo.swap(rest);
+            chain = fits;
         }
     }
     if (descs.empty()) return TN_OK;
